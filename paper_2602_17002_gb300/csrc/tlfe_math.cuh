@@ -5,17 +5,27 @@
 // the deformation gradient F = sum_i x_i h_i^T (Sec. 2.1) equals I + G with
 // G = sum_i u_i h_i^T. Strain-like quantities are formed from G directly so
 // that FP32 keeps its relative accuracy at small strain:
-//   E     = (G + G^T + G^T G) / 2
-//   b - I = G + G^T + G G^T
+//   B     = C - I = G + G^T + G^T G  (twice the Green strain)
 //   J - 1 = tr G + I2(G) + det G     (expansion of det(I + G))
-// The Mooney-Rivlin stress of App. C (Eq. mr_first_piola; neo-Hookean is
-// mu01 = 0) is used in the algebraically equal form
-//   P = [ 2 mu10 J^{-5/3} D + 2 mu01 J^{-7/3} dev(I1 b - b^2) + k (J - 1) I ] cof(F)
-// with cof(F) = J F^{-T}, D = dev(b - I) and, writing b = I + beta,
-//   dev(I1 b - b^2) = (1 + tr(beta)/3) D - dev(D D)
-// (I1 F - F C = (I1 b - b^2) F^{-T} and F = b F^{-T}), which needs no division
-// by J in the volumetric term and no cancellation of the identity in the
-// isochoric ones.
+// Every law is evaluated through its second Piola-Kirchhoff stress S, P = F S:
+// S and its derivative are symmetric (6 entries), the elastic and the viscous
+// part share one product with F, and the derivative along dF needs two 3x3
+// products, dP = dF S + F dS, with dS linear in dE = sym(F^T dF). With
+// P = A cof(F) (first Piola-Kirchhoff form) the neo-Hookean + Kelvin-Voigt
+// stress and its derivative took about 515 multiply-adds a point instead of
+// about 350.
+// Mooney-Rivlin (App. C, Eq. mr_first_piola; neo-Hookean is mu01 = 0):
+//   S = 2 mu10 J^{-2/3} (I - I1/3 C^{-1}) + 2 mu01 J^{-4/3} (I1 I - C - 2/3 I2 C^{-1})
+//       + k (J - 1) J C^{-1}
+// with C^{-1} = Q / J^2, Q = cof(C) = (1 + t) I - B + cof(B), t = tr B. The
+// isochoric brackets vanish at C = I; written in B they lose no digits there
+// (I2, I3: invariants of B; J^2 = 1 + t + I2 + I3):
+//   J^2 (I - I1/3 C^{-1}) = M = (1 + t/3) (B - cof B) - (t/3 + t^2/3 - I2 - I3) I
+//   J^2 (I1 I - C - 2/3 I2(C) C^{-1}) = M2
+//     = (1 + t/3 - I2/3 - I3) B - 2/3 (3 + 2t + I2) cof B
+//       + ((I2 + I3)(2 + t) - t/3 - t^2/3 - 2/3 I2 (1 + t)) I
+// so that S = alpha M + alpha2 M2 + beta Q with alpha = 2 mu10 J^{-8/3},
+// alpha2 = 2 mu01 J^{-10/3}, beta = k (J - 1) / J.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -51,34 +61,6 @@ template <typename R> struct Mat {
 
 template <typename R> __device__ __forceinline__ R tr3(const R A[9]) { return A[0] + A[4] + A[8]; }
 
-// cofactor matrix cof(F) (rows = cross products of the other two rows); equals J F^{-T}
-template <typename R> __device__ __forceinline__ void cof3(const R F[9], R C[9])
-{
-    C[0] = F[4] * F[8] - F[5] * F[7];
-    C[1] = F[5] * F[6] - F[3] * F[8];
-    C[2] = F[3] * F[7] - F[4] * F[6];
-    C[3] = F[7] * F[2] - F[8] * F[1];
-    C[4] = F[8] * F[0] - F[6] * F[2];
-    C[5] = F[6] * F[1] - F[7] * F[0];
-    C[6] = F[1] * F[5] - F[2] * F[4];
-    C[7] = F[2] * F[3] - F[0] * F[5];
-    C[8] = F[0] * F[4] - F[1] * F[3];
-}
-
-// directional derivative of cof at F along dF (cof is quadratic in F)
-template <typename R> __device__ __forceinline__ void dcof3(const R F[9], const R D[9], R C[9])
-{
-    C[0] = D[4] * F[8] + F[4] * D[8] - D[5] * F[7] - F[5] * D[7];
-    C[1] = D[5] * F[6] + F[5] * D[6] - D[3] * F[8] - F[3] * D[8];
-    C[2] = D[3] * F[7] + F[3] * D[7] - D[4] * F[6] - F[4] * D[6];
-    C[3] = D[7] * F[2] + F[7] * D[2] - D[8] * F[1] - F[8] * D[1];
-    C[4] = D[8] * F[0] + F[8] * D[0] - D[6] * F[2] - F[6] * D[2];
-    C[5] = D[6] * F[1] + F[6] * D[1] - D[7] * F[0] - F[7] * D[0];
-    C[6] = D[1] * F[5] + F[1] * D[5] - D[2] * F[4] - F[2] * D[4];
-    C[7] = D[2] * F[3] + F[2] * D[3] - D[0] * F[5] - F[0] * D[5];
-    C[8] = D[0] * F[4] + F[0] * D[4] - D[1] * F[3] - F[1] * D[3];
-}
-
 // R = A B
 template <typename R> __device__ __forceinline__ void mm3(const R A[9], const R B[9], R C[9])
 {
@@ -87,16 +69,6 @@ template <typename R> __device__ __forceinline__ void mm3(const R A[9], const R 
 #pragma unroll
         for (int b = 0; b < 3; ++b)
             C[a * 3 + b] = A[a * 3] * B[b] + A[a * 3 + 1] * B[3 + b] + A[a * 3 + 2] * B[6 + b];
-}
-
-// C += A B
-template <typename R> __device__ __forceinline__ void mm3_acc(const R A[9], const R B[9], R C[9])
-{
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-            C[a * 3 + b] += A[a * 3] * B[b] + A[a * 3 + 1] * B[3 + b] + A[a * 3 + 2] * B[6 + b];
 }
 
 // FP32 products with rows 0 and 1 paired in packed FP32x2 operations (one
@@ -115,33 +87,98 @@ __device__ __forceinline__ void mm3(const float A[9], const float B[9], float C[
         C[6 + b] = fmaf(A[8], B[6 + b], fmaf(A[7], B[3 + b], A[6] * B[b]));
     }
 }
-__device__ __forceinline__ void mm3_acc(const float A[9], const float B[9], float C[9])
+
+// Symmetric 3x3 matrices as 6 entries xx yy zz xy xz yz. Strain-like ones
+// (B, dE of a direction) that are summed with their transpose keep the
+// off-diagonal sums unhalved ("engineering" shear): entry xy of eng(A, B)
+// is (A^T B)_xy + (A^T B)_yx, the diagonal is that of A^T B.
+template <typename R> __device__ __forceinline__ void sym_eng(const R A[9], const R B[9], R e[6])
 {
-    const float2 a0 = make_float2(A[0], A[3]), a1 = make_float2(A[1], A[4]), a2 = make_float2(A[2], A[5]);
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        float2 q = __fmul2_rn(a0, make_float2(B[b], B[b]));
-        q = __ffma2_rn(a1, make_float2(B[3 + b], B[3 + b]), q);
-        q = __ffma2_rn(a2, make_float2(B[6 + b], B[6 + b]), q);
-        const float2 c = __fadd2_rn(make_float2(C[b], C[3 + b]), q);
-        C[b] = c.x;
-        C[3 + b] = c.y;
-        C[6 + b] += fmaf(A[8], B[6 + b], fmaf(A[7], B[3 + b], A[6] * B[b]));
-    }
+    for (int a = 0; a < 3; ++a) e[a] = A[a] * B[a] + A[3 + a] * B[3 + a] + A[6 + a] * B[6 + a];
+    e[3] = A[0] * B[1] + A[3] * B[4] + A[6] * B[7] + A[1] * B[0] + A[4] * B[3] + A[7] * B[6];
+    e[4] = A[0] * B[2] + A[3] * B[5] + A[6] * B[8] + A[2] * B[0] + A[5] * B[3] + A[8] * B[6];
+    e[5] = A[1] * B[2] + A[4] * B[5] + A[7] * B[8] + A[2] * B[1] + A[5] * B[4] + A[8] * B[7];
 }
 
-// sym(A^T B) = (A^T B + B^T A) / 2
-template <typename R> __device__ __forceinline__ void symAtB(const R A[9], const R B[9], R S[9])
+// S : e for a symmetric S and an engineering e (the doubled off-diagonals are in e)
+template <typename R> __device__ __forceinline__ R dot6(const R S[6], const R e[6])
+{
+    return S[0] * e[0] + S[1] * e[1] + S[2] * e[2] + S[3] * e[3] + S[4] * e[4] + S[5] * e[5];
+}
+
+// cofactors of a symmetric matrix
+template <typename R> __device__ __forceinline__ void cof6(const R B[6], R c[6])
+{
+    c[0] = B[1] * B[2] - B[5] * B[5];
+    c[1] = B[0] * B[2] - B[4] * B[4];
+    c[2] = B[0] * B[1] - B[3] * B[3];
+    c[3] = B[4] * B[5] - B[3] * B[2];
+    c[4] = B[3] * B[5] - B[4] * B[1];
+    c[5] = B[3] * B[4] - B[5] * B[0];
+}
+
+// derivative of cof6 at C along dC = 2 sym, given e = eng(F, dF) = (dE_xx, .., 2 dE_xy, ..):
+// diagonal entries halved (d/2), off-diagonal ones whole
+template <typename R> __device__ __forceinline__ void dcof6(const R C[6], const R e[6], R d[6])
+{
+    const R t0 = e[0] + e[0], t1 = e[1] + e[1], t2 = e[2] + e[2];
+    d[0] = C[1] * e[2] + C[2] * e[1] - C[5] * e[5];
+    d[1] = C[0] * e[2] + C[2] * e[0] - C[4] * e[4];
+    d[2] = C[0] * e[1] + C[1] * e[0] - C[3] * e[3];
+    d[3] = C[4] * e[5] + C[5] * e[4] - C[2] * e[3] - C[3] * t2;
+    d[4] = C[3] * e[5] + C[5] * e[3] - C[1] * e[4] - C[4] * t1;
+    d[5] = C[3] * e[4] + C[4] * e[3] - C[0] * e[5] - C[5] * t0;
+}
+
+// P = A S with S symmetric (6 entries)
+template <typename R> __device__ __forceinline__ void mm6(const R A[9], const R S[6], R P[9])
 {
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int a = 0; a < 3; ++a) {
+        P[a * 3 + 0] = A[a * 3] * S[0] + A[a * 3 + 1] * S[3] + A[a * 3 + 2] * S[4];
+        P[a * 3 + 1] = A[a * 3] * S[3] + A[a * 3 + 1] * S[1] + A[a * 3 + 2] * S[5];
+        P[a * 3 + 2] = A[a * 3] * S[4] + A[a * 3 + 1] * S[5] + A[a * 3 + 2] * S[2];
+    }
+}
+template <typename R> __device__ __forceinline__ void mm6_acc(const R A[9], const R S[6], R P[9])
+{
 #pragma unroll
-        for (int b = a; b < 3; ++b) {
-            R s = A[a] * B[b] + A[3 + a] * B[3 + b] + A[6 + a] * B[6 + b] + B[a] * A[b] +
-                  B[3 + a] * A[3 + b] + B[6 + a] * A[6 + b];
-            S[a * 3 + b] = R(0.5) * s;
-            S[b * 3 + a] = R(0.5) * s;
-        }
+    for (int a = 0; a < 3; ++a) {
+        P[a * 3 + 0] += A[a * 3] * S[0] + A[a * 3 + 1] * S[3] + A[a * 3 + 2] * S[4];
+        P[a * 3 + 1] += A[a * 3] * S[3] + A[a * 3 + 1] * S[1] + A[a * 3 + 2] * S[5];
+        P[a * 3 + 2] += A[a * 3] * S[4] + A[a * 3 + 1] * S[5] + A[a * 3 + 2] * S[2];
+    }
+}
+// FP32: rows 0 and 1 paired in packed FP32x2 operations (one issue slot for
+// two multiply-adds; broadcast and swapped operands are free)
+__device__ __forceinline__ void mm6(const float A[9], const float S[6], float P[9])
+{
+    const float2 a0 = make_float2(A[0], A[3]), a1 = make_float2(A[1], A[4]), a2 = make_float2(A[2], A[5]);
+    const float s[9] = {S[0], S[3], S[4], S[3], S[1], S[5], S[4], S[5], S[2]};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        float2 q = __fmul2_rn(a0, make_float2(s[b], s[b]));
+        q = __ffma2_rn(a1, make_float2(s[3 + b], s[3 + b]), q);
+        q = __ffma2_rn(a2, make_float2(s[6 + b], s[6 + b]), q);
+        P[b] = q.x;
+        P[3 + b] = q.y;
+        P[6 + b] = fmaf(A[8], s[6 + b], fmaf(A[7], s[3 + b], A[6] * s[b]));
+    }
+}
+__device__ __forceinline__ void mm6_acc(const float A[9], const float S[6], float P[9])
+{
+    const float2 a0 = make_float2(A[0], A[3]), a1 = make_float2(A[1], A[4]), a2 = make_float2(A[2], A[5]);
+    const float s[9] = {S[0], S[3], S[4], S[3], S[1], S[5], S[4], S[5], S[2]};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        float2 q = __ffma2_rn(a0, make_float2(s[b], s[b]), make_float2(P[b], P[3 + b]));
+        q = __ffma2_rn(a1, make_float2(s[3 + b], s[3 + b]), q);
+        q = __ffma2_rn(a2, make_float2(s[6 + b], s[6 + b]), q);
+        P[b] = q.x;
+        P[3 + b] = q.y;
+        P[6 + b] = fmaf(A[8], s[6 + b], fmaf(A[7], s[3 + b], fmaf(A[6], s[b], P[6 + b])));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -153,12 +190,14 @@ template <typename R> struct QP {
     R F[9];    // I + G
     R G[9];    // sum u_i h_i^T
     R Fd[9];   // sum udot_i h_i^T (valid when visc)
-    R S[9];    // SVK: elastic 2nd PK stress; MR / NH: A with P = A cof(F)
-    R Sv[9];   // viscous 2nd PK stress
-    R Cf[9];   // NH: cof(F)
-    R dev[9];  // MR / NH: D = dev(b - I)
-    R Jm1, J, Jm53, rJ;  // J - 1, J, J^{-5/3}, 1/J
-    R bt;      // MR: tr(b - I) / 3
+    R S[6];    // elastic second Piola-Kirchhoff stress
+    R Sv[6];   // viscous second Piola-Kirchhoff stress (valid when visc)
+    R B[6];    // C - I
+    R Q[6];    // MR / NH: cof(C)
+    R M[6];    // MR / NH: J^2 (I - I1/3 C^{-1})
+    R al, be;  // MR / NH: 2 mu10 J^{-8/3}, k (J - 1) / J
+    R rJ, r1, r2;  // MR / NH: 1 / J, J^{-1/3}, J^{-2/3}
+    R Jm1r;    // MR / NH: (J - 1) / J
     bool ok;
 };
 
@@ -166,11 +205,10 @@ template <typename R> __device__ __forceinline__ R rcbrt_(R x);
 template <> __device__ __forceinline__ float rcbrt_<float>(float x) { return rcbrtf(x); }
 template <> __device__ __forceinline__ double rcbrt_<double>(double x) { return rcbrt(x); }
 
-// Elastic + viscous stress. visc: whether Fd is meaningful and the material damped.
-// Returns P. Sets q.ok = false (and P = viscous part only) when the
-// neo-Hookean law meets J <= 0.
-template <typename R>
-__device__ __forceinline__ void stress(const Mat<R> &m, QP<R> &q, bool visc, R P[9])
+// Elastic and viscous stress state. visc: whether Fd is meaningful and the
+// material damped. Sets q.ok = false (and no elastic part) when the
+// neo-Hookean law meets J <= 0 or a J that is not a number.
+template <typename R> __device__ __forceinline__ void stress_state(const Mat<R> &m, QP<R> &q, bool visc)
 {
     const R *G = q.G;
 #pragma unroll
@@ -178,275 +216,257 @@ __device__ __forceinline__ void stress(const Mat<R> &m, QP<R> &q, bool visc, R P
     q.ok = true;
     if (visc) {
         // Edot = sym(Fd^T F); S^v = 2 mu_v Edot + lam_v tr(Edot) I  (Sec. 3.2.3)
-        R Ed[9];
-        symAtB(q.Fd, q.F, Ed);
-        const R t = tr3(Ed);
+        R e[6];
+        sym_eng(q.Fd, q.F, e);
+        const R i = m.lam_v * (e[0] + e[1] + e[2]);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) q.Sv[k] = R(2) * m.mu_v * Ed[k];
-        q.Sv[0] += m.lam_v * t;
-        q.Sv[4] += m.lam_v * t;
-        q.Sv[8] += m.lam_v * t;
+        for (int k = 0; k < 3; ++k) {
+            q.Sv[k] = R(2) * m.mu_v * e[k] + i;
+            q.Sv[3 + k] = m.mu_v * e[3 + k];
+        }
     }
+    // B = G + G^T + G^T G
+#pragma unroll
+    for (int a = 0; a < 3; ++a) q.B[a] = R(2) * G[4 * a] + G[a] * G[a] + G[3 + a] * G[3 + a] + G[6 + a] * G[6 + a];
+    q.B[3] = G[1] + G[3] + G[0] * G[1] + G[3] * G[4] + G[6] * G[7];
+    q.B[4] = G[2] + G[6] + G[0] * G[2] + G[3] * G[5] + G[6] * G[8];
+    q.B[5] = G[5] + G[7] + G[1] * G[2] + G[4] * G[5] + G[7] * G[8];
+    const R t = q.B[0] + q.B[1] + q.B[2];
     if (m.model == MODEL_SVK) {
-        // E = (G + G^T + G^T G)/2, S = lam tr(E) I + 2 mu E, P = F S  (App. C SVK)
-        R E[9];
+        // S = lam tr(E) I + 2 mu E  (App. C SVK)
+        const R i = R(0.5) * m.lam * t;
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = a; b < 3; ++b) {
-                R s = G[a * 3 + b] + G[b * 3 + a] + G[a] * G[b] + G[3 + a] * G[3 + b] + G[6 + a] * G[6 + b];
-                E[a * 3 + b] = R(0.5) * s;
-                E[b * 3 + a] = R(0.5) * s;
-            }
-        const R t = tr3(E);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) q.S[k] = R(2) * m.mu * E[k];
-        q.S[0] += m.lam * t;
-        q.S[4] += m.lam * t;
-        q.S[8] += m.lam * t;
-        if (visc) {
-            R St[9];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) St[k] = q.S[k] + q.Sv[k];
-            mm3(q.F, St, P);
-        } else {
-            mm3(q.F, q.S, P);
+        for (int k = 0; k < 3; ++k) {
+            q.S[k] = m.mu * q.B[k] + i;
+            q.S[3 + k] = m.mu * q.B[3 + k];
         }
         return;
     }
     // neo-Hookean: mu10 = mu/2, k = lam + 2 mu / 3
     const R third = R(1.0 / 3.0);
-    const R kb = m.lam + R(2) * third * m.mu;
-    const R I2 = G[0] * G[4] + G[4] * G[8] + G[0] * G[8] - G[1] * G[3] - G[5] * G[7] - G[2] * G[6];
-    const R dG = G[0] * (G[4] * G[8] - G[5] * G[7]) - G[1] * (G[3] * G[8] - G[5] * G[6]) +
-                 G[2] * (G[3] * G[7] - G[4] * G[6]);
-    q.Jm1 = tr3(G) + I2 + dG;
-    q.J = R(1) + q.Jm1;
-    if (!(q.J > R(0))) {
+    const R c0 = G[4] * G[8] - G[5] * G[7], c1 = G[5] * G[6] - G[3] * G[8], c2 = G[3] * G[7] - G[4] * G[6];
+    const R dG = G[0] * c0 + G[1] * c1 + G[2] * c2;
+    const R I2G = c0 + (G[0] * G[4] - G[1] * G[3]) + (G[0] * G[8] - G[2] * G[6]);
+    const R Jm1 = tr3(G) + I2G + dG;
+    const R J = R(1) + Jm1;
+    if (!(J > R(0))) {
         q.ok = false;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) P[k] = R(0);
-        if (visc) mm3(q.F, q.Sv, P);
+        for (int k = 0; k < 6; ++k) q.S[k] = q.Q[k] = q.M[k] = q.B[k] = R(0);
+        q.al = q.be = q.rJ = q.r1 = q.r2 = q.Jm1r = R(0);
         return;
     }
-    const R r = rcbrt_<R>(q.J);
-    const R r2 = r * r;
-    const R r3 = r2 * r;  // 1/J
-    q.Jm53 = r3 * r2;
-    q.rJ = r3;
-    // b - I = G + G^T + G G^T
-    R bt = R(0);
+    const R r = rcbrt_<R>(J);
+    q.r1 = r;
+    q.r2 = r * r;
+    q.rJ = q.r2 * r;
+    const R rD = q.rJ * q.rJ;  // J^{-2}
+    q.Jm1r = Jm1 * q.rJ;
+    q.al = (m.mu - R(2) * m.mu01) * (rD * q.r2);
+    q.be = (m.lam + R(2) * third * m.mu) * q.Jm1r;
+    R cB[6];
+    cof6(q.B, cB);
+    const R I2 = cB[0] + cB[1] + cB[2];
+    const R I3 = q.B[0] * cB[0] + q.B[3] * cB[3] + q.B[4] * cB[4];
+    const R s = R(1) + third * t;
+    const R iso = (I2 + I3) - third * t * (R(1) + t);
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = a; b < 3; ++b) {
-            R s = G[a * 3 + b] + G[b * 3 + a] + G[a * 3] * G[b * 3] + G[a * 3 + 1] * G[b * 3 + 1] +
-                  G[a * 3 + 2] * G[b * 3 + 2];
-            q.dev[a * 3 + b] = s;
-            q.dev[b * 3 + a] = s;
-        }
-    bt = tr3(q.dev) * third;
-    q.bt = bt;
-    q.dev[0] -= bt;
-    q.dev[4] -= bt;
-    q.dev[8] -= bt;
-    const R c1 = (m.mu - R(2) * m.mu01) * q.Jm53;  // 2 mu10 J^{-5/3}
-#pragma unroll
-    for (int k = 0; k < 9; ++k) q.S[k] = c1 * q.dev[k];
-    if (m.model == MODEL_MR) {
-        // + 2 mu01 J^{-7/3} [ (1 + tr(beta)/3) D - dev(D D) ]
-        const R c2 = R(2) * m.mu01 * q.Jm53 * q.Jm53 * q.J;
-        R DD[9];
-        mm3(q.dev, q.dev, DD);
-        const R t = tr3(DD) * third;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) q.S[k] += c2 * ((R(1) + bt) * q.dev[k] - DD[k]);
-        q.S[0] += c2 * t;
-        q.S[4] += c2 * t;
-        q.S[8] += c2 * t;
+    for (int k = 0; k < 6; ++k) {
+        const R bc = q.B[k] - cB[k];
+        q.Q[k] = k < 3 ? (R(1) + t) - bc : -bc;
+        q.M[k] = k < 3 ? s * bc + iso : s * bc;
+        q.S[k] = q.al * q.M[k] + q.be * q.Q[k];
     }
-    q.S[0] += kb * q.Jm1;
-    q.S[4] += kb * q.Jm1;
-    q.S[8] += kb * q.Jm1;
-    cof3(q.F, q.Cf);
-    mm3(q.S, q.Cf, P);
-    if (visc) mm3_acc(q.F, q.Sv, P);
+    if (m.model == MODEL_MR) {
+        const R a2 = R(2) * m.mu01 * rD * q.rJ * r;  // 2 mu01 J^{-10/3}
+        const R x1 = R(1) + third * (t - I2) - I3;
+        const R x2 = R(2) * third * (R(3) + R(2) * t + I2);
+        const R x0 = (I2 + I3) * (R(2) + t) - third * t * (R(1) + t) - R(2) * third * I2 * (R(1) + t);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const R M2 = x1 * q.B[k] - x2 * cB[k] + (k < 3 ? x0 : R(0));
+            q.S[k] += a2 * M2;
+        }
+    }
+}
+
+// first Piola-Kirchhoff stress of the state: F (S + S^v)
+template <typename R> __device__ __forceinline__ void first_piola(const QP<R> &q, bool visc, R P[9])
+{
+    R St[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) St[k] = visc ? q.S[k] + q.Sv[k] : q.S[k];
+    mm6(q.F, St, P);
+    if (!q.ok && !visc)  // an F that is not a number leaves no trace
+#pragma unroll
+        for (int k = 0; k < 9; ++k) P[k] = R(0);
+}
+
+template <typename R>
+__device__ __forceinline__ void stress(const Mat<R> &m, QP<R> &q, bool visc, R P[9])
+{
+    stress_state<R>(m, q, visc);
+    first_piola<R>(q, visc, P);
+}
+
+// c times the elastic derivative dS along e = eng(F, dF)
+template <typename R>
+__device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<R> &q, const R e[6], R c, R dS[6])
+{
+    const R trE = e[0] + e[1] + e[2];
+    if (m.model == MODEL_SVK) {
+        const R i = c * m.lam * trE, a = c * m.mu;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            dS[k] = R(2) * a * e[k] + i;
+            dS[3 + k] = a * e[3 + k];
+        }
+        return;
+    }
+    // S_iso = alpha M = mu J^{-2/3} (I - I1/3 C^{-1}), C^{-1} = Q / J^2, j = dJ / J = C^{-1} : dE:
+    //   dS_iso = -(2/3) j S_iso - mu J^{-2/3}/3 (2 tr dE C^{-1} + I1 dC^{-1})
+    //   d(k (J - 1) J C^{-1}) = k (2J - 1) J j C^{-1} + k (J - 1) J dC^{-1}
+    //   dC^{-1} = (dQ - 2 j Q) / J^2
+    const R third = R(1.0 / 3.0);
+    const R t = q.B[0] + q.B[1] + q.B[2];
+    const R rD = q.rJ * q.rJ;
+    const R j = dot6(q.Q, e) * rD;
+    const R aI = third * q.al * (R(3) + t);  // alpha I1 / 3
+    const R kb = m.lam + R(2) * third * m.mu;
+    const R xM = c * (R(-2) * third * q.al * j);
+    const R xQ = c * (j * (kb - q.be + R(2) * aI) - R(2) * third * q.al * trE);
+    const R xd = c * (q.be - aI);
+    R C[6], dQ[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) C[k] = k < 3 ? R(1) + q.B[k] : q.B[k];
+    dcof6(C, e, dQ);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) dS[k] = xM * q.M[k] + xQ * q.Q[k] + (k < 3 ? R(2) * xd : xd) * dQ[k];
+    if (m.model == MODEL_MR) {
+        // S2 = a2 M2, a2 = 2 mu01 J^{-10/3}: dS2 = -(10/3) j S2 + a2 dM2
+        R cB[6];
+        cof6(q.B, cB);
+        const R I2 = cB[0] + cB[1] + cB[2];
+        const R I3 = q.B[0] * cB[0] + q.B[3] * cB[3] + q.B[4] * cB[4];
+        const R x1 = R(1) + third * (t - I2) - I3;
+        const R x2 = R(2) * third * (R(3) + R(2) * t + I2);
+        const R x0 = (I2 + I3) * (R(2) + t) - third * t * (R(1) + t) - R(2) * third * I2 * (R(1) + t);
+        const R a2 = R(2) * m.mu01 * rD * q.rJ * q.r1;  // 2 mu01 J^{-10/3}
+        // invariants of B along dB = 2 dE
+        R dcB[6];
+        dcof6(q.B, e, dcB);  // diagonal halved
+        const R dt = R(2) * trE;
+        const R dI2 = R(2) * (dcB[0] + dcB[1] + dcB[2]);
+        const R dI3 = R(2) * (cB[0] * e[0] + cB[1] * e[1] + cB[2] * e[2] + cB[3] * e[3] + cB[4] * e[4] + cB[5] * e[5]);
+        const R dx1 = third * (dt - dI2) - dI3;
+        const R dx2 = R(2) * third * (R(2) * dt + dI2);
+        const R dx0 = (dI2 + dI3) * (R(2) + t) + (I2 + I3) * dt - third * dt * (R(1) + R(2) * t) -
+                      R(2) * third * (dI2 * (R(1) + t) + I2 * dt);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const R M2 = x1 * q.B[k] - x2 * cB[k] + (k < 3 ? x0 : R(0));
+            const R dB = k < 3 ? R(2) * e[k] : e[k];
+            const R dc = k < 3 ? R(2) * dcB[k] : dcB[k];
+            const R dM2 = dx1 * q.B[k] + x1 * dB - dx2 * cB[k] - x2 * dc + (k < 3 ? dx0 : R(0));
+            dS[k] += c * a2 * (dM2 - R(10) * third * j * M2);
+        }
+    }
 }
 
 // Directional derivative of P along (dF, dFd):
-//   dP = D_F P^e[dF] + (position-side viscous terms, if visc_pos)
-//        + D_Fd P^v[dFd]  (if has_dFd)
-// cK scales everything depending on dF, cC everything depending on dFd.
-// sym_only drops the viscous stiffness K^v (the non-symmetric part).
+//   dP = D_F P^e[dF] + (position-side viscous terms, if visc and not sym_only)
+//        + D_Fd P^v[dFd]
+// with dF = dFd the given direction; cK scales everything depending on dF, cC
+// everything depending on dFd. sym_only drops the viscous stiffness K^v (the
+// non-symmetric part).
 template <typename R>
 __device__ __forceinline__ void dstress(const Mat<R> &m, const QP<R> &q, bool visc, const R dF[9],
                                         R cK, R cC, bool sym_only, R dP[9])
 {
-#pragma unroll
-    for (int k = 0; k < 9; ++k) dP[k] = R(0);
+    R e[6], T[6];
+    sym_eng(q.F, dF, e);
     if (cK != R(0)) {
-        if (m.model == MODEL_SVK) {
-            // dE = sym(F^T dF); dS = lam tr(dE) I + 2 mu dE; dP = dF S + F dS
-            R dE[9], dS[9];
-            symAtB(q.F, dF, dE);
-            const R t = tr3(dE);
+        R Sk[6];
+        dS_elastic<R>(m, q, e, cK, T);
+        const bool vk = visc && !sym_only;
+        if (vk) {  // position-side viscous derivative: dEdot = sym(Fd^T dF)
+            R ev[6];
+            sym_eng(q.Fd, dF, ev);
+            const R a = cK * m.mu_v, i = cK * m.lam_v * (ev[0] + ev[1] + ev[2]);
 #pragma unroll
-            for (int k = 0; k < 9; ++k) dS[k] = R(2) * m.mu * dE[k];
-            dS[0] += m.lam * t;
-            dS[4] += m.lam * t;
-            dS[8] += m.lam * t;
-            mm3_acc(dF, q.S, dP);
-            mm3_acc(q.F, dS, dP);
-        } else if (q.ok) {
-            const R third = R(1.0 / 3.0);
-            const R kb = m.lam + R(2) * third * m.mu;
-            // dJ = cof(F) : dF
-            R dJ = R(0);
-#pragma unroll
-            for (int k = 0; k < 9; ++k) dJ += q.Cf[k] * dF[k];
-            // d(b - I) = dF + dF^T + dF G^T + G dF^T
-            R db[9];
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int b = a; b < 3; ++b) {
-                    R s = dF[a * 3 + b] + dF[b * 3 + a] + dF[a * 3] * q.G[b * 3] +
-                          dF[a * 3 + 1] * q.G[b * 3 + 1] + dF[a * 3 + 2] * q.G[b * 3 + 2] +
-                          q.G[a * 3] * dF[b * 3] + q.G[a * 3 + 1] * dF[b * 3 + 1] +
-                          q.G[a * 3 + 2] * dF[b * 3 + 2];
-                    db[a * 3 + b] = s;
-                    db[b * 3 + a] = s;
-                }
-            const R dbt = tr3(db) * third;
-            db[0] -= dbt;
-            db[4] -= dbt;
-            db[8] -= dbt;
-            const R dJm53 = R(-5.0 / 3.0) * q.Jm53 * dJ * q.rJ;
-            const R mu2 = m.mu - R(2) * m.mu01;  // 2 mu10
-            R dA[9];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) dA[k] = mu2 * (dJm53 * q.dev[k] + q.Jm53 * db[k]);
-            if (m.model == MODEL_MR) {
-                // d{ c2 [ (1 + bt) D - dev(D D) ] }, c2 = 2 mu01 J^{-7/3}
-                const R c2 = R(2) * m.mu01 * q.Jm53 * q.Jm53 * q.J;
-                const R dc2 = R(-7.0 / 3.0) * c2 * dJ * q.rJ;
-                R DD[9], dDD[9];
-                mm3(q.dev, q.dev, DD);
-                mm3(db, q.dev, dDD);
-                mm3_acc(q.dev, db, dDD);
-                const R t = tr3(DD) * third, dt = tr3(dDD) * third;
-#pragma unroll
-                for (int k = 0; k < 9; ++k)
-                    dA[k] += dc2 * ((R(1) + q.bt) * q.dev[k] - DD[k]) +
-                             c2 * (dbt * q.dev[k] + (R(1) + q.bt) * db[k] - dDD[k]);
-                const R iso = dc2 * t + c2 * dt;
-                dA[0] += iso;
-                dA[4] += iso;
-                dA[8] += iso;
+            for (int k = 0; k < 3; ++k) {
+                T[k] += R(2) * a * ev[k] + i;
+                T[3 + k] += a * ev[3 + k];
             }
-            dA[0] += kb * dJ;
-            dA[4] += kb * dJ;
-            dA[8] += kb * dJ;
-            R dC[9];
-            dcof3(q.F, dF, dC);
-            mm3_acc(dA, q.Cf, dP);
-            mm3_acc(q.S, dC, dP);
-        }
-        if (visc && !sym_only) {
-            mm3_acc(dF, q.Sv, dP);  // q.S holds the elastic part only, for both laws
-            // F dS^v with dEdot = sym(Fd^T dF)
-            R dE[9], dS[9];
-            symAtB(q.Fd, dF, dE);
-            const R t = tr3(dE);
-#pragma unroll
-            for (int k = 0; k < 9; ++k) dS[k] = R(2) * m.mu_v * dE[k];
-            dS[0] += m.lam_v * t;
-            dS[4] += m.lam_v * t;
-            dS[8] += m.lam_v * t;
-            mm3_acc(q.F, dS, dP);
         }
 #pragma unroll
-        for (int k = 0; k < 9; ++k) dP[k] *= cK;
-    }
-    if (cC != R(0) && (m.mu_v != R(0) || m.lam_v != R(0))) {
-        // velocity direction: dEdot = sym(F^T dFd), dP = F dS^v
-        R dE[9], dS[9], T[9];
-        symAtB(q.F, dF, dE);
-        const R t = tr3(dE);
+        for (int k = 0; k < 6; ++k) Sk[k] = cK * (vk ? q.S[k] + q.Sv[k] : q.S[k]);
+        mm6(dF, Sk, dP);
+    } else {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) dS[k] = R(2) * m.mu_v * dE[k];
-        dS[0] += m.lam_v * t;
-        dS[4] += m.lam_v * t;
-        dS[8] += m.lam_v * t;
-        mm3(q.F, dS, T);
+        for (int k = 0; k < 6; ++k) T[k] = R(0);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) dP[k] += cC * T[k];
+        for (int k = 0; k < 9; ++k) dP[k] = R(0);
     }
+    if (cC != R(0)) {  // velocity direction: dEdot = sym(F^T dFd)
+        const R a = cC * m.mu_v, i = cC * m.lam_v * (e[0] + e[1] + e[2]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            T[k] += R(2) * a * e[k] + i;
+            T[3 + k] += a * e[3 + k];
+        }
+    }
+    mm6_acc(q.F, T, dP);
+    if (!q.ok && !(visc && !sym_only) && !(cC != R(0) && (m.mu_v != R(0) || m.lam_v != R(0))))
+#pragma unroll
+        for (int k = 0; k < 9; ++k) dP[k] = R(0);
 }
 
 // Adjoint of the stress map at one point against a cotangent Gh (=sum r_i h_i^T):
 //   gF  = (dP/dF)^T [Gh]  (elastic part self-adjoint; viscous part explicit)
 //   gFd = (dP/dFd)^T [Gh]
-//   gmu = dP/dmu : Gh, glam = dP/dlam : Gh
+//   gmu = dP/dmu : Gh, glam = dP/dlam : Gh, contracted as dS/dmu : sym(F^T Gh)
 template <typename R>
 __device__ __forceinline__ void astress(const Mat<R> &m, const QP<R> &q, bool visc, const R Gh[9],
                                         R gF[9], R gFd[9], R &gmu, R &glam)
 {
-    dstress<R>(m, q, false, Gh, R(1), R(0), true, gF);
+    R e[6], T[6], St[6];
+    sym_eng(q.F, Gh, e);
+    dS_elastic<R>(m, q, e, R(1), T);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) gFd[k] = R(0);
+    for (int k = 0; k < 6; ++k) St[k] = visc ? q.S[k] + q.Sv[k] : q.S[k];
+    mm6(Gh, St, gF);
+    mm6_acc(q.F, T, gF);
+    const R trE = e[0] + e[1] + e[2];
     if (visc) {
-        // L = (F S^v) : Gh.  Sbar = sym(F^T Gh), Ebar = 2 mu_v Sbar + lam_v tr(Sbar) I
-        // dL/dF = Gh S^v + Fd Ebar,  dL/dFd = F Ebar
-        R Sb[9], Eb[9];
-        symAtB(q.F, Gh, Sb);
-        const R t = tr3(Sb);
+        // L = (F S^v) : Gh, Ebar = 2 mu_v sym(F^T Gh) + lam_v tr I:
+        // dL/dF = Gh S^v + Fd Ebar, dL/dFd = F Ebar
+        R Eb[6];
+        const R i = m.lam_v * trE;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) Eb[k] = R(2) * m.mu_v * Sb[k];
-        Eb[0] += m.lam_v * t;
-        Eb[4] += m.lam_v * t;
-        Eb[8] += m.lam_v * t;
-        mm3_acc(Gh, q.Sv, gF);
-        mm3_acc(q.Fd, Eb, gF);
-        mm3(q.F, Eb, gFd);
+        for (int k = 0; k < 3; ++k) {
+            Eb[k] = R(2) * m.mu_v * e[k] + i;
+            Eb[3 + k] = m.mu_v * e[3 + k];
+        }
+        mm6_acc(q.Fd, Eb, gF);
+        mm6(q.F, Eb, gFd);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            gFd[k] = R(0);
+            if (!q.ok) gF[k] = R(0);
+        }
     }
-    gmu = R(0);
-    glam = R(0);
     if (m.model == MODEL_SVK) {
-        // dP/dlam = tr(E) F, dP/dmu = 2 F E ; E recovered from S = lam trE I + 2 mu E
-        // is ill-posed when mu = 0, so recompute E from G.
-        R E[9];
-        const R *G = q.G;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b)
-                E[a * 3 + b] = R(0.5) * (G[a * 3 + b] + G[b * 3 + a] + G[a] * G[b] + G[3 + a] * G[3 + b] +
-                                         G[6 + a] * G[6 + b]);
-        R FE[9];
-        mm3(q.F, E, FE);
-        const R t = tr3(E);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            gmu += R(2) * FE[k] * Gh[k];
-            glam += t * q.F[k] * Gh[k];
-        }
-    } else if (q.ok) {
-        // P = [(mu - 2 mu01) J^{-5/3} D + 2 mu01 J^{-7/3} D2 + (lam + 2mu/3)(J-1) I] cof with
-        // mu01 held fixed: dP/dmu = [J^{-5/3} D + 2/3 (J-1) I] cof, dP/dlam = (J-1) cof
-        R Bm[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) Bm[k] = q.Jm53 * q.dev[k];
-        Bm[0] += R(2.0 / 3.0) * q.Jm1;
-        Bm[4] += R(2.0 / 3.0) * q.Jm1;
-        Bm[8] += R(2.0 / 3.0) * q.Jm1;
-        R Pm[9];
-        mm3(Bm, q.Cf, Pm);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            gmu += Pm[k] * Gh[k];
-            glam += q.Jm1 * q.Cf[k] * Gh[k];
-        }
+        // dS/dlam = tr(E) I, dS/dmu = 2 E = B
+        gmu = dot6(q.B, e);
+        glam = R(0.5) * (q.B[0] + q.B[1] + q.B[2]) * trE;
+    } else {
+        // dS/dmu = J^{-8/3} M + 2/3 (J - 1)/J Q (mu01 held fixed), dS/dlam = (J - 1)/J Q
+        const R gq = q.Jm1r * dot6(q.Q, e);
+        const R g = q.rJ * q.rJ * q.r2 * dot6(q.M, e) + R(2.0 / 3.0) * gq;
+        gmu = q.ok ? g : R(0);
+        glam = q.ok ? gq : R(0);
     }
 }
 
