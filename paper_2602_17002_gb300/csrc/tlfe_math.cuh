@@ -25,7 +25,11 @@
 //     = (1 + t/3 - I2/3 - I3) B - 2/3 (3 + 2t + I2) cof B
 //       + ((I2 + I3)(2 + t) - t/3 - t^2/3 - 2/3 I2 (1 + t)) I
 // so that S = alpha M + alpha2 M2 + beta Q with alpha = 2 mu10 J^{-8/3},
-// alpha2 = 2 mu01 J^{-10/3}, beta = k (J - 1) / J.
+// alpha2 = 2 mu01 J^{-10/3}, beta = k (J - 1) / J. M and Q are both sums of I
+// and N = B - cof(B): with s = 1 + t/3 and i = I2 + I3 - t (1 + t)/3,
+//   M = s N + i I, Q = (1 + t) I - N,
+//   S = (alpha s - beta) N + (alpha i + beta (1 + t)) I      (+ alpha2 M2),
+// and the same holds for the parts of dS that M and Q enter: neither is formed.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -193,11 +197,11 @@ template <typename R> struct QP {
     R S[6];    // elastic second Piola-Kirchhoff stress
     R Sv[6];   // viscous second Piola-Kirchhoff stress (valid when visc)
     R B[6];    // C - I
-    R Q[6];    // MR / NH: cof(C)
-    R M[6];    // MR / NH: J^2 (I - I1/3 C^{-1})
-    R al, be;  // MR / NH: 2 mu10 J^{-8/3}, k (J - 1) / J
-    R rJ, r1, r2;  // MR / NH: 1 / J, J^{-1/3}, J^{-2/3}
-    R Jm1r;    // MR / NH: (J - 1) / J
+    R N[6];    // MR / NH: B - cof(B)
+    // MR / NH: alpha, alpha s - beta, and the scalars of the header comment
+    R al, c1, s, i, t1;   // t1 = 1 + t
+    R rD, rJ, r1;         // J^{-2}, 1/J, J^{-1/3}
+    R Jm1r;               // (J - 1) / J
     bool ok;
 };
 
@@ -252,36 +256,36 @@ template <typename R> __device__ __forceinline__ void stress_state(const Mat<R> 
     if (!(J > R(0))) {
         q.ok = false;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) q.S[k] = q.Q[k] = q.M[k] = q.B[k] = R(0);
-        q.al = q.be = q.rJ = q.r1 = q.r2 = q.Jm1r = R(0);
+        for (int k = 0; k < 6; ++k) q.S[k] = q.N[k] = q.B[k] = R(0);
+        q.al = q.c1 = q.s = q.i = q.t1 = q.rD = q.rJ = q.r1 = q.Jm1r = R(0);
         return;
     }
-    const R r = rcbrt_<R>(J);
+    const R r = rcbrt_<R>(J), r2 = r * r;
     q.r1 = r;
-    q.r2 = r * r;
-    q.rJ = q.r2 * r;
-    const R rD = q.rJ * q.rJ;  // J^{-2}
+    q.rJ = r2 * r;
+    q.rD = q.rJ * q.rJ;
     q.Jm1r = Jm1 * q.rJ;
-    q.al = (m.mu - R(2) * m.mu01) * (rD * q.r2);
-    q.be = (m.lam + R(2) * third * m.mu) * q.Jm1r;
+    q.al = (m.mu - R(2) * m.mu01) * (q.rD * r2);
+    const R be = (m.lam + R(2) * third * m.mu) * q.Jm1r;
     R cB[6];
     cof6(q.B, cB);
     const R I2 = cB[0] + cB[1] + cB[2];
     const R I3 = q.B[0] * cB[0] + q.B[3] * cB[3] + q.B[4] * cB[4];
-    const R s = R(1) + third * t;
-    const R iso = (I2 + I3) - third * t * (R(1) + t);
+    q.t1 = R(1) + t;
+    q.s = R(1) + third * t;
+    q.i = (I2 + I3) - third * t * q.t1;
+    q.c1 = q.al * q.s - be;
+    const R iso = q.al * q.i + be * q.t1;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        const R bc = q.B[k] - cB[k];
-        q.Q[k] = k < 3 ? (R(1) + t) - bc : -bc;
-        q.M[k] = k < 3 ? s * bc + iso : s * bc;
-        q.S[k] = q.al * q.M[k] + q.be * q.Q[k];
+        q.N[k] = q.B[k] - cB[k];
+        q.S[k] = k < 3 ? q.c1 * q.N[k] + iso : q.c1 * q.N[k];
     }
     if (m.model == MODEL_MR) {
-        const R a2 = R(2) * m.mu01 * rD * q.rJ * r;  // 2 mu01 J^{-10/3}
+        const R a2 = R(2) * m.mu01 * q.rD * q.rJ * r;  // 2 mu01 J^{-10/3}
         const R x1 = R(1) + third * (t - I2) - I3;
         const R x2 = R(2) * third * (R(3) + R(2) * t + I2);
-        const R x0 = (I2 + I3) * (R(2) + t) - third * t * (R(1) + t) - R(2) * third * I2 * (R(1) + t);
+        const R x0 = (I2 + I3) * (R(2) + t) - third * t * q.t1 - R(2) * third * I2 * q.t1;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const R M2 = x1 * q.B[k] - x2 * cB[k] + (k < 3 ? x0 : R(0));
@@ -328,22 +332,24 @@ __device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<R> &q, cons
     //   d(k (J - 1) J C^{-1}) = k (2J - 1) J j C^{-1} + k (J - 1) J dC^{-1}
     //   dC^{-1} = (dQ - 2 j Q) / J^2
     const R third = R(1.0 / 3.0);
-    const R t = q.B[0] + q.B[1] + q.B[2];
-    const R rD = q.rJ * q.rJ;
-    const R j = dot6(q.Q, e) * rD;
-    const R aI = third * q.al * (R(3) + t);  // alpha I1 / 3
     const R kb = m.lam + R(2) * third * m.mu;
-    const R xM = c * (R(-2) * third * q.al * j);
-    const R xQ = c * (j * (kb - q.be + R(2) * aI) - R(2) * third * q.al * trE);
-    const R xd = c * (q.be - aI);
+    const R as = q.al * q.s;  // alpha I1 / 3; beta = as - c1
+    const R QE = q.t1 * trE - dot6(q.N, e);
+    const R j = QE * q.rD;
+    const R a23 = c * R(2) * third * q.al;
+    const R xM = -a23 * j;
+    const R xQ = c * j * (kb + as + q.c1) - a23 * trE;
+    const R xd = -c * q.c1;
+    const R y1 = xM * q.s - xQ, y0 = xM * q.i + xQ * q.t1;
     R C[6], dQ[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) C[k] = k < 3 ? R(1) + q.B[k] : q.B[k];
     dcof6(C, e, dQ);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) dS[k] = xM * q.M[k] + xQ * q.Q[k] + (k < 3 ? R(2) * xd : xd) * dQ[k];
+    for (int k = 0; k < 6; ++k) dS[k] = k < 3 ? y1 * q.N[k] + (R(2) * xd * dQ[k] + y0) : y1 * q.N[k] + xd * dQ[k];
     if (m.model == MODEL_MR) {
         // S2 = a2 M2, a2 = 2 mu01 J^{-10/3}: dS2 = -(10/3) j S2 + a2 dM2
+        const R t = q.B[0] + q.B[1] + q.B[2];
         R cB[6];
         cof6(q.B, cB);
         const R I2 = cB[0] + cB[1] + cB[2];
@@ -351,7 +357,7 @@ __device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<R> &q, cons
         const R x1 = R(1) + third * (t - I2) - I3;
         const R x2 = R(2) * third * (R(3) + R(2) * t + I2);
         const R x0 = (I2 + I3) * (R(2) + t) - third * t * (R(1) + t) - R(2) * third * I2 * (R(1) + t);
-        const R a2 = R(2) * m.mu01 * rD * q.rJ * q.r1;  // 2 mu01 J^{-10/3}
+        const R a2 = R(2) * m.mu01 * q.rD * q.rJ * q.r1;  // 2 mu01 J^{-10/3}
         // invariants of B along dB = 2 dE
         R dcB[6];
         dcof6(q.B, e, dcB);  // diagonal halved
@@ -463,8 +469,9 @@ __device__ __forceinline__ void astress(const Mat<R> &m, const QP<R> &q, bool vi
         glam = R(0.5) * (q.B[0] + q.B[1] + q.B[2]) * trE;
     } else {
         // dS/dmu = J^{-8/3} M + 2/3 (J - 1)/J Q (mu01 held fixed), dS/dlam = (J - 1)/J Q
-        const R gq = q.Jm1r * dot6(q.Q, e);
-        const R g = q.rJ * q.rJ * q.r2 * dot6(q.M, e) + R(2.0 / 3.0) * gq;
+        const R NE = dot6(q.N, e);
+        const R gq = q.Jm1r * (q.t1 * trE - NE);
+        const R g = q.rD * q.r1 * q.r1 * (q.s * NE + q.i * trE) + R(2.0 / 3.0) * gq;
         gmu = q.ok ? g : R(0);
         glam = q.ok ? gq : R(0);
     }
