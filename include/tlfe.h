@@ -195,7 +195,7 @@ typedef struct {
                                      over the tile kernels' loads; 1 = free of bank conflicts */
     int32_t force_matvec_fused;   /* 1: tlfe_force_matvec and tlfe_step_host (with f and y requested)
                                      evaluate the force and the operator product in one pass per element
-                                     block and law (FP32 meshes of T4, T10 and H8 blocks, neither
+                                     block and law (FP32 meshes of T4, T10 and H8 blocks, FP64 meshes of affine T10 blocks, neither
                                      operation on the persistent launch; tlfe_autotune keeps the faster
                                      of one fused pass and two passes); 0: two passes */
     int64_t stream_bytes_force_matvec;  /* algorithmic bytes of that fused pass (u, udot, v read once; f, y) */
@@ -312,7 +312,7 @@ tlfe_status tlfe_tangent_matvec(tlfe_mesh *mesh, const void *u_dev, const void *
  * the first after tlfe_autotune, tlfe_set_launch_mode or the first
  * tlfe_set_elem_mu_lambda) evaluates directly and captures the same launches
  * on a stream of its own; later calls with the same arguments replay that
- * graph on `stream`. On an FP32 mesh of T4, T10 and H8 blocks the two
+ * graph on `stream`. On an FP32 mesh of T4, T10 and H8 blocks, or an FP64 mesh of affine T10 blocks, the two
  * operations run as one pass per element block and law, which gathers the
  * nodal inputs and forms F, Fdot and the stress once for both outputs
  * (tlfe_mesh_info.force_matvec_fused says whether it does; tlfe_autotune keeps

@@ -1192,9 +1192,11 @@ static tlfe_status launch_block(tlfe_mesh *m, int bi, KParams<R> p, cudaStream_t
         }
         p.tile_chunk = ls.chunk;
         p.rmw_scatter = m->scatter == TLFE_SCATTER_COLOR ? 1 : 0;
-        // one warp per tile (per element on the warp-per-element path) at a
-        // time, persistent over the resident warps
-        const int units = wpe_path(B.et, B.use_affine) ? tiles * TILE : tiles;
+        // one warp per tile (per element on the warp-per-element path, one CTA
+        // per tile on the point-per-warp path) at a time, persistent over the
+        // resident warps
+        const int units = wpe_path(B.et, B.use_affine) ? tiles * TILE
+                                                       : (pw_path(B.et, B.use_affine, OP, sizeof(R) == 4) ? tiles * ls.wpb : tiles);
         const int warps = std::min(units, std::max(1, ls.resident / ls.wpb) * ls.wpb * m->n_sm);
         const int grid = std::max(1, (warps + ls.wpb - 1) / ls.wpb);
         cudaError_t e = launch_op<OP, R>(B.et, B.nq, p, grid, ls.wpb, s);
@@ -1372,13 +1374,15 @@ tlfe_status run_op(tlfe_mesh *m, const void *u, const void *ud, const void *v, v
 
 // The fused force + operator-product pass (OP_FM) exists for the tile
 // kernels of FP32 T4, T10 and H8 blocks (not for Q27, whose affine blocks run
-// the warp-per-element kernels); it replaces the two per-pass launches where
+// the warp-per-element kernels) and for FP64 affine T10 blocks (the
+// point-per-warp kernels); it replaces the two per-pass launches where
 // neither operation runs as the persistent launch.
 static bool fm_kernels(const tlfe_mesh *m)
 {
-    if (m->precision != TLFE_FP32) return false;
-    for (const BlockStore &B : m->blocks)
-        if (B.n_elem > 0 && B.et == ET_Q27) return false;
+    for (const BlockStore &B : m->blocks) {
+        if (B.n_elem == 0) continue;
+        if (m->precision == TLFE_FP32 ? B.et == ET_Q27 : !pw_path(B.et, B.use_affine, OP_FM, false)) return false;
+    }
     return true;
 }
 
@@ -1390,7 +1394,9 @@ bool fm_eligible(const tlfe_mesh *m)
 tlfe_status force_matvec_op(tlfe_mesh *m, const void *u, const void *ud, const void *v, double aM, double aK,
                             double aC, void *f, void *y, cudaStream_t s)
 {
-    if (fm_eligible(m)) return run_op<OP_FM, float>(m, u, ud, v, f, y, nullptr, aM, aK, aC, 0, s);
+    if (fm_eligible(m))
+        return m->precision == TLFE_FP32 ? run_op<OP_FM, float>(m, u, ud, v, f, y, nullptr, aM, aK, aC, 0, s)
+                                         : run_op<OP_FM, double>(m, u, ud, v, f, y, nullptr, aM, aK, aC, 0, s);
     tlfe_status st;
     if (m->precision == TLFE_FP32) {
         st = run_op<OP_FORCE, float>(m, u, ud, nullptr, f, nullptr, nullptr, 0, 1, 0, 0, s);
@@ -1555,27 +1561,27 @@ static tlfe_status tune_all(tlfe_mesh *m, const double *u, const void *ud, const
             st = tune_fused<OP_FORCE>(m, p, s, e0, e1);
             if (st == TLFE_OK && v) st = tune_fused<OP_MATVEC>(m, p, s, e0, e1);
         }
-        // the fused force + operator-product pass: its own schedules, then one
-        // fused pass against the two passes (with their tuned schedules) on
-        // the caller's inputs; the faster is kept
-        if (st == TLFE_OK && v && fm_kernels(m)) {
-            m->fm_on = 1;
-            for (int bi = 0; bi < (int)m->blocks.size() && st == TLFE_OK; ++bi)
-                if (m->blocks[bi].n_elem > 0) st = tune_block<OP_FM, R>(m, bi, p, s, e0, e1);
-            if (st == TLFE_OK && fm_eligible(m)) {
-                float t_fm = 0.f, t_two = 0.f;
-                st = time_median3([&]() { return run_op<OP_FM, float>(m, u, ud, v, o0, o1, nullptr, 0, 1, 1, 0, s); },
-                                  s, e0, e1, &t_fm);
-                if (st == TLFE_OK)
-                    st = time_median3(
-                        [&]() {
-                            tlfe_status s2 = run_op<OP_FORCE, float>(m, u, ud, nullptr, o0, nullptr, nullptr, 0, 1, 0, 0, s);
-                            return s2 != TLFE_OK ? s2
-                                                 : run_op<OP_MATVEC, float>(m, u, ud, v, o1, nullptr, nullptr, 0, 1, 1, 0, s);
-                        },
-                        s, e0, e1, &t_two);
-                if (st == TLFE_OK) m->fm_on = t_fm <= t_two ? 1 : 0;
-            }
+    }
+    // the fused force + operator-product pass: its own schedules, then one
+    // fused pass against the two passes (with their tuned schedules) on
+    // the caller's inputs; the faster is kept
+    if (st == TLFE_OK && v && fm_kernels(m)) {
+        m->fm_on = 1;
+        for (int bi = 0; bi < (int)m->blocks.size() && st == TLFE_OK; ++bi)
+            if (m->blocks[bi].n_elem > 0) st = tune_block<OP_FM, R>(m, bi, p, s, e0, e1);
+        if (st == TLFE_OK && fm_eligible(m)) {
+            float t_fm = 0.f, t_two = 0.f;
+            st = time_median3([&]() { return run_op<OP_FM, R>(m, u, ud, v, o0, o1, nullptr, 0, 1, 1, 0, s); }, s, e0,
+                              e1, &t_fm);
+            if (st == TLFE_OK)
+                st = time_median3(
+                    [&]() {
+                        tlfe_status s2 = run_op<OP_FORCE, R>(m, u, ud, nullptr, o0, nullptr, nullptr, 0, 1, 0, 0, s);
+                        return s2 != TLFE_OK ? s2
+                                             : run_op<OP_MATVEC, R>(m, u, ud, v, o1, nullptr, nullptr, 0, 1, 1, 0, s);
+                    },
+                    s, e0, e1, &t_two);
+            if (st == TLFE_OK) m->fm_on = t_fm <= t_two ? 1 : 0;
         }
     }
     cudaStreamSynchronize(s);
@@ -1595,6 +1601,7 @@ template tlfe_status run_op<OP_DIAG, float>(tlfe_mesh *, const void *, const voi
 template tlfe_status run_op<OP_DIAG, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
 template tlfe_status run_op<OP_VJP, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
 template tlfe_status run_op<OP_VJP, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
+template tlfe_status run_op<OP_FM, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
 template tlfe_status run_op<OP_FM, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
 
 }  // namespace tlfe

@@ -39,7 +39,9 @@
 // flight, each by the parity of its barrier's one outstanding phase, and
 // returns.
 // Affine Q27 blocks do not come here: they run the warp-per-element kernels
-// of k_wpe.cuh (kernel_for / smem_for below dispatch on wpe_path).
+// of k_wpe.cuh; nor do FP64 operations on affine T10 blocks (but the
+// diagonal), which run one warp per quadrature point (k_pw.cuh). kernel_for /
+// smem_for below dispatch on wpe_path and pw_path.
 #pragma once
 
 #include <string>
@@ -1120,6 +1122,7 @@ __global__ void __launch_bounds__(128, min_ctas<ET, R, OP, AFF, MAT>()) k_elem(c
 
 }  // namespace tlfe
 
+#include "k_pw.cuh"
 #include "k_wpe.cuh"
 
 namespace tlfe {
@@ -1159,7 +1162,9 @@ template <int OP, typename R> static void (*kernel_for(int et, int nq, bool aff,
     } else {
         if (wpe_path(et, aff)) return wpe_kernel_for<OP, R>(mat);
     }
-    return aff ? kernel_for_m<OP, R, true>(et, nq, mat) : kernel_for_m<OP, R, false>(et, nq, mat);
+    if (pw_path(et, aff, OP, sizeof(R) == 4)) return pw_kernel_for<OP, R>(nq);
+    if constexpr (OP == OP_FM && sizeof(R) != 4) return nullptr;
+    else return aff ? kernel_for_m<OP, R, true>(et, nq, mat) : kernel_for_m<OP, R, false>(et, nq, mat);
 }
 
 template <int OP, typename R, bool AFF> size_t smem_for_(int et, int umax, int meta_bytes, int wpb)
@@ -1170,14 +1175,16 @@ template <int OP, typename R, bool AFF> size_t smem_for_(int et, int umax, int m
     if (et == ET_Q27 && OP != OP_FM) return elem_smem_bytes<ET_Q27, R, OP, AFF>(umax, meta_bytes, wpb);
     return 0;
 }
-template <int OP, typename R> size_t smem_for(int et, int umax, int meta_bytes, int wpb, bool aff)
+template <int OP, typename R> size_t smem_for(int et, int nq, int umax, int meta_bytes, int wpb, bool aff)
 {
     if (wpe_path(et, aff)) return OP == OP_FM ? 0 : wpe_smem_bytes<R>(wpb);
+    if (pw_path(et, aff, OP, sizeof(R) == 4)) return pw_smem_for<OP>(nq, umax, meta_bytes);
     return aff ? smem_for_<OP, R, true>(et, umax, meta_bytes, wpb) : smem_for_<OP, R, false>(et, umax, meta_bytes, wpb);
 }
 
 // resident warps per SM for the best CTA size among 4, 2 and 1 warps, or for
-// the CTA size *wpb_io when it is positive on entry
+// the CTA size *wpb_io when it is positive on entry. The point-per-warp
+// kernels have one CTA size, nq warps, which answers for 4.
 template <int OP, typename R>
 int occupancy_op(int et, int nq, bool aff, int mat, int umax, int meta_bytes, int *wpb_io, std::string *why)
 {
@@ -1188,10 +1195,13 @@ int occupancy_op(int et, int nq, bool aff, int mat, int umax, int meta_bytes, in
         *why = "no kernel for this element type and quadrature size";
         return 0;
     }
+    const bool pw = pw_path(et, aff, OP, sizeof(R) == 4);
     int best = 0;
-    for (int wpb : {4, 2, 1}) {
-        if (only > 0 && wpb != only) continue;
-        const size_t smem = smem_for<OP, R>(et, umax, meta_bytes, wpb, aff);
+    for (int size : {4, 2, 1}) {
+        if (only > 0 && size != only && !(pw && only == nq)) continue;
+        if (pw && size != 4) continue;
+        const int wpb = pw ? nq : size;
+        const size_t smem = smem_for<OP, R>(et, nq, umax, meta_bytes, wpb, aff);
         if (smem > 227 * 1024) continue;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int nb = 0;
@@ -1219,7 +1229,7 @@ cudaError_t launch_op(int et, int nq, const KParams<R> &p, int grid, int wpb, cu
     const bool aff = p.aff != nullptr;
     void (*kern)(const KParams<R>) = kernel_for<OP, R>(et, nq, aff, p.mat_mode);
     if (!kern) return cudaErrorInvalidValue;
-    const size_t smem = smem_for<OP, R>(et, p.umax, p.meta_bytes, wpb, aff);
+    const size_t smem = smem_for<OP, R>(et, nq, p.umax, p.meta_bytes, wpb, aff);
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     kern<<<grid, 32 * wpb, smem, s>>>(p);

@@ -28,6 +28,13 @@ constexpr int AFF_ROWS = 10;  // affine record rows per tile: J^{-1} (9, row-maj
 // lanes over points then nodes); every other block runs one thread per element
 __host__ __device__ inline bool wpe_path(int et, bool aff) { return et == ET_Q27 && aff; }
 
+// FP64 operations but the diagonal on affine T10 blocks run one CTA per tile
+// and one warp per quadrature point (k_pw.cuh)
+__host__ __device__ constexpr bool pw_path(int et, bool aff, int op, bool fp32)
+{
+    return et == ET_T10 && aff && op != OP_DIAG && !fp32;
+}
+
 // values per node held in a warp's shared-memory patch: inputs (u, udot
 // [, v or cotangent]) then outputs (one array, two for the adjoint)
 __host__ __device__ constexpr int op_in_fields(int op) { return (op == OP_MATVEC || op == OP_VJP || op == OP_FM) ? 9 : 6; }
