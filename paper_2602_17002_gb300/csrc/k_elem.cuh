@@ -29,11 +29,11 @@
 //   - each lane evaluates F = I + sum_i u_i h_i^T per quadrature point and the
 //     stress, its directional derivative, its adjoint or the diagonal moduli,
 //     accumulating its element vector sum_q w_q J_p (.) h_iq in registers;
-//   - element vectors go to conflict-free shared slots [i * 32 + lane]; one
-//     lane per unique node sums that node's slots (a node-to-slot list built
-//     at mesh creation) and adds the sum to the global array with one atomic
-//     per component (a plain read-add-write in colour passes, where no two
-//     elements of a launch share a node).
+//   - element vectors go to shared slots in node-sorted positions (a list
+//     built at mesh creation); one lane per unique node sums that node's slots
+//     and adds the sum to the global array with one atomic per component (a
+//     plain read-add-write in colour passes, where no two elements of a launch
+//     share a node).
 // Every mbarrier wait is bounded; on timeout the kernel latches ST_TIMEOUT in
 // the status word, waits (again bounded) for the copies it still has in
 // flight, each by the parity of its barrier's one outstanding phase, and
@@ -179,16 +179,34 @@ template <typename R> struct AffRec {
     static constexpr uint32_t BYTES = ROWS * 32 * sizeof(R);  // multiple of 16
 };
 
+// element-vector slots of a tile. Wide slots (FP32, but for the diagonal and
+// for T4 with one output field) hold the vectors of all output fields, one
+// 16-byte slot (x, y, z of the first field, x of the second) and for two
+// fields one 8-byte slot (y, z of the second) per position; the others one
+// field at a time, [position][3]. The T4 force alone is slower with wide slots
+// (34.2 against 32.8 us on 849k elements): its four positions a lane leave no
+// instructions to save against the larger slots' bank conflicts.
+template <int ET, typename R, int OP> __host__ __device__ constexpr bool wide_slots()
+{
+    return sizeof(R) == 4 && OP != OP_DIAG && (ET != ET_T4 || OpFields<OP>::NFO == 2);
+}
+template <int ET, typename R, int OP> __host__ __device__ constexpr size_t slot_bytes()
+{
+    const size_t n = (size_t)Elem<ET>::NPE * 32;
+    if (wide_slots<ET, R, OP>()) return n * (OpFields<OP>::NFO == 2 ? 24 : 16);
+    return n * 3 * sizeof(R);
+}
+
 // shared memory of one warp: slice ring (isoparametric path only), two
 // metadata buffers (each followed, on the affine path, by the tile's affine
 // record), and a work area holding first the node patch [umax][REC] and later
-// the element-vector slots [npe * 32][3] of one output field; rounded up to
-// 128 bytes so that every bulk-copy destination stays 16-byte aligned
+// the element-vector slots; rounded up to 128 bytes so that every bulk-copy
+// destination stays 16-byte aligned
 template <int ET, typename R, int OP, bool AFF>
 __host__ __device__ constexpr size_t warp_region_bytes(int umax, int meta_bytes)
 {
     const size_t patch = (size_t)umax * Rec<OP, R>::REC * sizeof(R);
-    const size_t slots = (size_t)Elem<ET>::NPE * 32 * 3 * sizeof(R);  // one output field at a time
+    const size_t slots = slot_bytes<ET, R, OP>();
     const size_t ring = AFF ? 0 : (size_t)NSLICE * Slice<ET, R>::BYTES;
     const size_t mrec = (size_t)meta_bytes + (AFF ? AffRec<R>::BYTES : 0);
     return (ring + 2 * mrec + (patch > slots ? patch : slots) + 127) / 128 * 128;
@@ -999,27 +1017,108 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
         const int nbad = __reduce_add_sync(0xffffffffu, bad);
         if (lane == 0 && nbad) atomicAdd(p.status + ST_INVERTED, nbad);
 
-        // ---- per output field: each lane writes its element vector into the
-        // node-sorted position array (the patch is dead now), then one lane per
-        // unique node sums that node's contiguous positions and adds the sum
-        // to the global array. The sorted scatter stores the sum as the tile's
-        // partial instead (word 1 of the record: the tile's first partial
-        // position); it runs as its own copy of the loop, so that the adding
-        // path compiles as it does without it.
+        // ---- each lane writes its element vector into the node-sorted position
+        // array (the patch is dead now), then one lane per unique node sums that
+        // node's contiguous positions and adds the sum to the global array. The
+        // sorted scatter stores the sum as the tile's partial instead (word 1 of
+        // the record: the tile's first partial position); it runs as its own copy
+        // of the loop, so that the adding path compiles as it does without it.
+        // Wide slots: one walk over the positions sums every field, 2 shared
+        // loads and 3 packed additions a position of two fields where one walk
+        // per field over [position][3] took 6 and 6 and twice the loop around
+        // them, and 2 stores instead of 6 (beam step of 480k T10 273.6 -> 262.7
+        // us, 40-body batch 339 -> 317).
+        if constexpr (wide_slots<ET, R, OP>()) {
+            float4 *sA = reinterpret_cast<float4 *>(work);
+            float2 *sB = reinterpret_cast<float2 *>(sA + NPE * 32);
+            __syncwarp();
+            if (valid) {
+#pragma unroll
+                for (int i = 0; i < NPE; ++i) {
+                    const int ps = (int)bounds_clamp(spos[i * 32 + lane], NPE * 32, p.status);
+                    sA[ps] = make_float4(ap0[i].x, ap0[i].y, acc0[i][2], TWO ? ap1[i].x : 0.f);
+                    if constexpr (TWO) sB[ps] = make_float2(ap1[i].y, acc1[i][2]);
+                }
+            }
+            __syncwarp();
+            auto node_sums = [&](int kk, float4 &a, float2 &b) {
+                const int s0 = (int)bounds_clamp(soff[kk], NPE * 32 + 1, p.status);
+                const int s1e = (int)bounds_clamp(soff[kk + 1], NPE * 32 + 1, p.status);
+                float2 xy = make_float2(0.f, 0.f), zx = xy;
+                b = xy;
+                for (int sb = s0; sb < s1e; sb += 4) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (sb + j < s1e) {
+                            const float4 v = sA[sb + j];
+                            xy = add2(xy, make_float2(v.x, v.y));
+                            if constexpr (TWO) {
+                                zx = add2(zx, make_float2(v.z, v.w));
+                                b = add2(b, sB[sb + j]);
+                            } else {
+                                zx.x += v.z;
+                            }
+                        }
+                }
+                a = make_float4(xy.x, xy.y, zx.x, zx.y);
+            };
+            if (p.part0) {
+                const int64_t P0 = reinterpret_cast<const int32_t *>(M)[1];
+                for (int kk = lane; kk < U; kk += 32) {
+                    if (!bounds_ok(P0 + kk, p.n_part, p.status)) continue;
+                    float4 a;
+                    float2 b;
+                    node_sums(kk, a, b);
+                    R *d0 = p.part0 + (P0 + kk) * 3;
+                    d0[0] = a.x;
+                    d0[1] = a.y;
+                    d0[2] = a.z;
+                    if constexpr (TWO) {
+                        R *d1 = p.part1 + (P0 + kk) * 3;
+                        d1[0] = a.w;
+                        d1[1] = b.x;
+                        d1[2] = b.y;
+                    }
+                }
+            } else {
+                for (int kk = lane; kk < U; kk += 32) {
+                    const int64_t n = bounds_clamp(nodes[kk], p.n_nodes, p.status);
+                    float4 a;
+                    float2 b;
+                    node_sums(kk, a, b);
+                    R *o0 = p.out0 + 3 * n, *o1 = TWO ? p.out1 + 3 * n : nullptr;
+                    if (p.rmw_scatter) {
+                        o0[0] += a.x;
+                        o0[1] += a.y;
+                        o0[2] += a.z;
+                        if constexpr (TWO) {
+                            o1[0] += a.w;
+                            o1[1] += b.x;
+                            o1[2] += b.y;
+                        }
+                    } else {
+                        atomicAdd(o0, a.x);
+                        atomicAdd(o0 + 1, a.y);
+                        atomicAdd(o0 + 2, a.z);
+                        if constexpr (TWO) {
+                            atomicAdd(o1, a.w);
+                            atomicAdd(o1 + 1, b.x);
+                            atomicAdd(o1 + 2, b.y);
+                        }
+                    }
+                }
+            }
+        } else {
         auto slots_in = [&](int fo) {
             __syncwarp();
             if (valid) {
 #pragma unroll
                 for (int i = 0; i < NPE; ++i) {
                     const int ps = (int)bounds_clamp(spos[i * 32 + lane], NPE * 32, p.status);
-                    if constexpr (PKA) {
-                        const float2 a01 = fo == 0 ? ap0[i] : ap1[i];
-                        work[ps * 3] = a01.x;
-                        work[ps * 3 + 1] = a01.y;
-                        work[ps * 3 + 2] = fo == 0 ? acc0[i][2] : acc1[i][2];
-                    } else {
 #pragma unroll
-                        for (int d = 0; d < 3; ++d) work[ps * 3 + d] = fo == 0 ? acc0[i][d] : acc1[i][d];
+                    for (int d = 0; d < 3; ++d) {
+                        if constexpr (PKA) work[ps * 3 + d] = d == 0 ? ap0[i].x : (d == 1 ? ap0[i].y : acc0[i][2]);
+                        else work[ps * 3 + d] = fo == 0 ? acc0[i][d] : acc1[i][d];
                     }
                 }
             }
@@ -1074,6 +1173,7 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
                     }
                 }
             }
+        }
         }
         __syncwarp();
     }
