@@ -787,6 +787,16 @@ static tlfe_status build_block(tlfe_mesh *m, const tlfe_mesh_desc *d, int bi, in
     return TLFE_OK;
 }
 
+// material mode of pass c of block B: the pass's law, with the viscous term
+// when a velocity is given and an element of the pass is damped
+static int pass_mat_mode(const BlockStore &B, int c, bool have_ud)
+{
+    const bool visc = have_ud && B.pass_visc[c];
+    if (B.pass_model[c] == MODEL_NH) return visc ? MAT_NH_KV : MAT_NH;
+    if (B.pass_model[c] == MODEL_SVK) return visc ? MAT_SVK_KV : MAT_SVK;
+    return MAT_ANY;
+}
+
 // Work items of the fused launch: the passes the fused kernels cover (FP32,
 // atomic or sorted scatter, affine T4 / T10 / H8 tile blocks), when there are
 // at least two. Each pass is cut into runs of tiles of about equal work
@@ -841,8 +851,10 @@ static tlfe_status build_fused_plan(tlfe_mesh *m)
         for (auto &pc : passes) {
             const BlockStore &B = m->blocks[pc.first];
             const int code = fused_code(B.et, B.nq);
-            w = std::max(w, o == 0 ? fused_warp_region<float, OP_FORCE>(code, B.umax, B.meta_bytes)
-                                   : fused_warp_region<float, OP_MATVEC>(code, B.umax, B.meta_bytes));
+            // with a velocity given or not: the mode without one needs no more
+            const int mat = pass_mat_mode(B, pc.second, true);
+            w = std::max(w, o == 0 ? fused_warp_region<float, OP_FORCE>(code, B.umax, B.meta_bytes, mat)
+                                   : fused_warp_region<float, OP_MATVEC>(code, B.umax, B.meta_bytes, mat));
         }
         fp->wreg[o] = w;
     }
@@ -1109,16 +1121,6 @@ template <typename R> static const Mat<R> *mats_of(const tlfe_mesh *m);
 template <> const Mat<float> *mats_of<float>(const tlfe_mesh *m) { return m->d_mats_f; }
 template <> const Mat<double> *mats_of<double>(const tlfe_mesh *m) { return m->d_mats_d; }
 
-// material mode of pass c of block B: the pass's law, with the viscous term
-// when a velocity is given and an element of the pass is damped
-static int pass_mat_mode(const BlockStore &B, int c, bool have_ud)
-{
-    const bool visc = have_ud && B.pass_visc[c];
-    if (B.pass_model[c] == MODEL_NH) return visc ? MAT_NH_KV : MAT_NH;
-    if (B.pass_model[c] == MODEL_SVK) return visc ? MAT_SVK_KV : MAT_SVK;
-    return MAT_ANY;
-}
-
 // fill the block-independent fields of an element launch for block B
 template <typename R> static void block_params(tlfe_mesh *m, const BlockStore &B, KParams<R> &p)
 {
@@ -1148,9 +1150,12 @@ template <typename R> static void block_params(tlfe_mesh *m, const BlockStore &B
     p.n_elem_block = B.n_elem;
 }
 
-// the launch schedule of (OP, block bi): from the cache, else from the occupancy API
+// the launch schedule of (OP, block bi): from the cache, else from the
+// occupancy API. A mass term takes shared memory on the T10 path, so it has
+// its own count of resident warps, at the CTA size and tile assignment of the
+// schedule without one (tuned, where the autotuner ran).
 template <int OP, typename R>
-static tlfe_status block_sched(tlfe_mesh *m, int bi, int mat, LaunchSched *out)
+static tlfe_status block_sched(tlfe_mesh *m, int bi, int mat, bool mass, LaunchSched *out)
 {
     const BlockStore &B = m->blocks[bi];
     const auto key = std::make_tuple(OP, bi, mat, (int)sizeof(R));
@@ -1159,11 +1164,22 @@ static tlfe_status block_sched(tlfe_mesh *m, int bi, int mat, LaunchSched *out)
         std::string why;
         LaunchSched ls;
         ls.wpb = 0;  // best CTA size
-        ls.resident = occupancy_op<OP, R>(B.et, B.nq, B.use_affine, mat, B.umax, B.meta_bytes, &ls.wpb, &why);
+        ls.resident = occupancy_op<OP, R>(B.et, B.nq, B.use_affine, mat, false, B.umax, B.meta_bytes, &ls.wpb, &why);
         if (ls.resident <= 0) return fail(TLFE_E_UNSUPPORTED, "element kernel cannot be made resident: " + why);
         it = m->sched.emplace(key, ls).first;
     }
     *out = it->second;
+    if (mass) {
+        if (it->second.resident_mass <= 0) {
+            std::string why;
+            int wpb = it->second.wpb;
+            it->second.resident_mass =
+                occupancy_op<OP, R>(B.et, B.nq, B.use_affine, mat, true, B.umax, B.meta_bytes, &wpb, &why);
+            if (it->second.resident_mass <= 0)
+                return fail(TLFE_E_UNSUPPORTED, "element kernel cannot be made resident: " + why);
+        }
+        out->resident = it->second.resident_mass;
+    }
     return TLFE_OK;
 }
 
@@ -1187,7 +1203,7 @@ static tlfe_status launch_block(tlfe_mesh *m, int bi, KParams<R> p, cudaStream_t
         if (fixed) {
             ls = *fixed;
         } else {
-            tlfe_status st = block_sched<OP, R>(m, bi, p.mat_mode, &ls);
+            tlfe_status st = block_sched<OP, R>(m, bi, p.mat_mode, p.aM != R(0), &ls);
             if (st != TLFE_OK) return st;
         }
         p.tile_chunk = ls.chunk;
@@ -1430,7 +1446,7 @@ static tlfe_status tune_block(tlfe_mesh *m, int bi, KParams<R> p, cudaStream_t s
             std::string why;
             LaunchSched ls;
             ls.wpb = wpb;
-            ls.resident = occupancy_op<OP, R>(B.et, B.nq, B.use_affine, mat, B.umax, B.meta_bytes, &ls.wpb, &why);
+            ls.resident = occupancy_op<OP, R>(B.et, B.nq, B.use_affine, mat, p.aM != R(0), B.umax, B.meta_bytes, &ls.wpb, &why);
             if (ls.resident <= 0) continue;
             for (int chunk : {0, 1}) {
                 ls.chunk = chunk;

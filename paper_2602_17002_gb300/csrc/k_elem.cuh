@@ -45,7 +45,10 @@
 #pragma once
 
 #include <string>
+#include <type_traits>
 
+#include "k_h8.cuh"
+#include "k_t10.cuh"
 #include "tlfe_elem.cuh"
 #include "tlfe_internal.h"
 
@@ -158,6 +161,20 @@ __device__ __forceinline__ float4 lds4_volatile(const float *p)
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(smem_u32(p)));
     return v;
 }
+// loads of a tile's tables straight from global memory, issued where they stand
+// (volatile): their latency overlaps what follows up to their first use
+__device__ __forceinline__ int ldg_u16_volatile(const uint16_t *p)
+{
+    unsigned short v;
+    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return (int)v;
+}
+__device__ __forceinline__ float ldg_f32_volatile(const float *p)
+{
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ int lds_u16_volatile(const uint16_t *p)
 {
     unsigned short v;
@@ -197,27 +214,68 @@ template <int ET, typename R, int OP> __host__ __device__ constexpr size_t slot_
     return n * 3 * sizeof(R);
 }
 
+// FP32 affine T10 blocks run the point records of k_t10.cuh (all but the
+// diagonal): per lane the gradients of the fields at four points, u, udot
+// where the material mode is damped (or not known) and the direction
+template <typename R> __host__ __device__ constexpr bool t10_path(int et, int op, bool aff)
+{
+    return sizeof(R) == 4 && et == ET_T10 && aff && op != OP_DIAG;
+}
+__host__ __device__ constexpr bool mat_damped(int mat) { return mat == MAT_ANY || mat == MAT_NH_KV || mat == MAT_SVK_KV; }
+__host__ __device__ constexpr int t10_fields(int op, int mat) { return op_in_fields(op) / 3 - (mat_damped(mat) ? 0 : 1); }
+
+// FP32 affine H8 blocks run on the coefficients of the trilinear fields
+// (k_h8.cuh), all but the diagonal: per lane 7 x 3 values a field, and the sum
+// of the direction's nodal values for the mass term
+template <typename R> __host__ __device__ constexpr bool h8_path(int et, int op, bool aff)
+{
+    return sizeof(R) == 4 && et == ET_H8 && aff && op != OP_DIAG;
+}
+// whether its points are evaluated two at a time: where the state of two
+// points and the accumulators fit the registers
+__host__ __device__ constexpr bool h8_pairs(int op, int mat) { return mat != MAT_ANY && (op == OP_FORCE || (op == OP_MATVEC && mat == MAT_SVK)); }
+
+// T10 and H8 blocks on those paths read the per-lane tables of a tile (local
+// indices, slot positions, affine record) once each, straight from global
+// memory: of the metadata record only the head (unique-node count, element
+// ids, node list) and the node offsets at its end go through shared memory
+template <typename R> __host__ __device__ constexpr bool column_path(int et, int op, bool aff)
+{
+    return t10_path<R>(et, op, aff) || h8_path<R>(et, op, aff);
+}
+__host__ __device__ constexpr int meta_head_bytes(int umaxp) { return 16 + 128 + 4 * umaxp; }
+__host__ __device__ constexpr int meta_lane_bytes(int npe) { return 2 * npe * 32 * 2; }  // local indices, positions
+
 // shared memory of one warp: slice ring (isoparametric path only), two
 // metadata buffers (each followed, on the affine path, by the tile's affine
 // record), and a work area holding first the node patch [umax][REC] and later
 // the element-vector slots; rounded up to 128 bytes so that every bulk-copy
-// destination stays 16-byte aligned
+// destination stays 16-byte aligned. On the T10 path the work area also holds,
+// between the two, the lanes' J^{-1} [9][32], their point records [2][9 fields][32] float2 and, with
+// a mass term (`mass`), behind them the lanes' mass vectors [30][32]; on the
+// H8 path the lanes' J^{-1} and coefficients.
 template <int ET, typename R, int OP, bool AFF>
-__host__ __device__ constexpr size_t warp_region_bytes(int umax, int meta_bytes)
+__host__ __device__ constexpr size_t warp_region_bytes(int umax, int meta_bytes, int mat, bool mass)
 {
     const size_t patch = (size_t)umax * Rec<OP, R>::REC * sizeof(R);
     const size_t slots = slot_bytes<ET, R, OP>();
     const size_t ring = AFF ? 0 : (size_t)NSLICE * Slice<ET, R>::BYTES;
-    const size_t mrec = (size_t)meta_bytes + (AFF ? AffRec<R>::BYTES : 0);
-    return (ring + 2 * mrec + (patch > slots ? patch : slots) + 127) / 128 * 128;
+    const size_t mrec = column_path<R>(ET, OP, AFF) ? (size_t)meta_bytes - meta_lane_bytes(Elem<ET>::NPE)
+                                                    : (size_t)meta_bytes + (AFF ? AffRec<R>::BYTES : 0);
+    size_t work = patch > slots ? patch : slots;
+    if (t10_path<R>(ET, OP, AFF)) {
+        const size_t rec = ((size_t)9 + 4 * 9 * t10_fields(OP, mat) + (mass ? 30 : 0)) * 32 * sizeof(R);
+        work = work > rec ? work : rec;
+    }
+    if (h8_path<R>(ET, OP, AFF)) {
+        const size_t c = ((size_t)9 + 21 * t10_fields(OP, mat) + 3) * 32 * sizeof(R);
+        work = work > c ? work : c;
+    }
+    return (ring + 2 * mrec + work + 127) / 128 * 128;
 }
 
 // dynamic shared memory of one CTA with `wpb` warps (mbarriers, then the warp regions)
-template <int ET, typename R, int OP, bool AFF>
-__host__ __device__ constexpr size_t elem_smem_bytes(int umax, int meta_bytes, int wpb)
-{
-    return 128 + (size_t)wpb * warp_region_bytes<ET, R, OP, AFF>(umax, meta_bytes);
-}
+constexpr size_t cta_smem_bytes(size_t region, int wpb) { return 128 + (size_t)wpb * region; }
 
 // 3-vectors at compile-time offsets of a 16-byte-aligned shared record, with
 // the widest aligned vector accesses the offset allows
@@ -323,6 +381,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 template <int ET, typename R, int OP, bool AFF, int MAT> constexpr int min_ctas()
 {
     if (sizeof(R) != 4 || ET == ET_Q27) return 1;
+    if (t10_path<R>(ET, OP, AFF) || h8_path<R>(ET, OP, AFF)) return OP == OP_FORCE ? 4 : (MAT == MAT_ANY ? 2 : 3);
     if (OP == OP_VJP || OP == OP_FM) {
         const bool fits = ET == ET_T4 || MAT == MAT_NH_KV || MAT == MAT_SVK || (MAT == MAT_SVK_KV && AFF) ||
                           (ET == ET_H8 && MAT != MAT_ANY);
@@ -360,6 +419,9 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
     constexpr int ROWS = SL::ROWS;
     using PG = ParentGrad<ET, NQ, R>;
     constexpr uint32_t AB = AFF ? AffRec<R>::BYTES : 0;
+    constexpr bool T10R = t10_path<R>(ET, OP, AFF);    // point records (k_t10.cuh)
+    constexpr bool H8C = h8_path<R>(ET, OP, AFF);      // trilinear coefficients (k_h8.cuh)
+    constexpr bool LANECOL = T10R || H8C;  // the lane keeps its fields in its own shared column
     constexpr bool PF_EARLY = AFF && OP != OP_VJP;  // where the next tile's L2 prefetch goes (see prefetch_next)
     constexpr bool PF_NONE = AFF && OP == OP_VJP;
     constexpr bool LI_REREAD = OP == OP_FORCE || OP == OP_VJP || OP == OP_FM;
@@ -374,7 +436,8 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
     const int lane = threadIdx.x & 31;
     const int MB = p.meta_bytes;
     uint64_t *mbar = bar + NSLICE;
-    const size_t MRB = (size_t)MB + AB;                        // metadata (+ affine) record bytes
+    const int HB = meta_head_bytes(p.umaxp), TB = MB - HB - meta_lane_bytes(NPE);  // head, node offsets
+    const size_t MRB = LANECOL ? (size_t)(HB + TB) : (size_t)MB + AB;  // bytes of a metadata buffer
     unsigned char *ring = wbase;
     unsigned char *mbuf = wbase + (AFF ? 0 : NSLICE * SL::BYTES);  // [2][MB + AB]
     R *work = reinterpret_cast<R *>(mbuf + 2 * MRB);           // patch [umax][REC], later slots
@@ -394,8 +457,14 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
         const int t = t0 + k * tstep;
         unsigned char *dst = mbuf + (size_t)(k & 1) * MRB;
         mbar_arrive_expect_tx(mbar + (k & 1), (uint32_t)MRB);
-        bulk_g2s(dst, p.meta + (size_t)t * MB, (uint32_t)MB, mbar + (k & 1));
-        if constexpr (AFF) bulk_g2s(dst + MB, p.aff + (size_t)t * AffRec<R>::ROWS * 32, AB, mbar + (k & 1));
+        const unsigned char *src = p.meta + (size_t)t * MB;
+        if constexpr (LANECOL) {
+            bulk_g2s(dst, src, (uint32_t)HB, mbar + (k & 1));
+            bulk_g2s(dst + HB, src + (MB - TB), (uint32_t)TB, mbar + (k & 1));
+        } else {
+            bulk_g2s(dst, src, (uint32_t)MB, mbar + (k & 1));
+        }
+        if constexpr (AFF && !LANECOL) bulk_g2s(dst + MB, p.aff + (size_t)t * AffRec<R>::ROWS * 32, AB, mbar + (k & 1));
     };
     if (lane == 0) {
         if (n_my > 0) issue_meta(0);
@@ -430,9 +499,11 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
         const int U = (int)bounds_clamp(*reinterpret_cast<const int32_t *>(M), (int64_t)p.umax + 1, p.status);
         const int e = reinterpret_cast<const int32_t *>(M + 16)[lane];
         const int32_t *nodes = reinterpret_cast<const int32_t *>(M + 16 + 128);
-        const uint16_t *mlidx = reinterpret_cast<const uint16_t *>(M + 16 + 128 + 4 * p.umaxp);
+        // in shared memory, or in global memory on the column paths
+        const uint16_t *mlidx = reinterpret_cast<const uint16_t *>((LANECOL ? p.meta + (size_t)t * MB : M) + HB);
         const uint16_t *spos = mlidx + NPE * 32;  // slot (i, lane) -> node-sorted position
-        const uint16_t *soff = spos + NPE * 32;   // positions of unique node kk: [soff[kk], soff[kk + 1])
+        // positions of unique node kk: [soff[kk], soff[kk + 1])
+        const uint16_t *soff = LANECOL ? reinterpret_cast<const uint16_t *>(M + HB) : spos + NPE * 32;
 
         // ---- gather the tile's nodal inputs into the patch, one record per
         // unique node: every lane issues asynchronous copies (cp.async) for all
@@ -466,6 +537,16 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
             }
         }
         cp_async_commit();
+        int li[NPE];
+        R Ji[9], detJ = R(0);  // affine path: J^{-1} and det J of this lane's element (Sec. 6, affine case)
+        if constexpr (LANECOL) {  // in flight together with the gather
+#pragma unroll
+            for (int i = 0; i < NPE; ++i) li[i] = ldg_u16_volatile(mlidx + i * 32 + lane);
+            const R *A = p.aff + (size_t)t * AFF_ROWS * 32 + lane;
+#pragma unroll
+            for (int r = 0; r < 9; ++r) Ji[r] = ldg_f32_volatile(A + r * 32);
+            detJ = ldg_f32_volatile(A + 9 * 32);
+        }
         cp_async_wait<0>();
         if constexpr (PK) {
             for (int kk = lane; kk < U; kk += 32) {
@@ -480,9 +561,8 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
                 *reinterpret_cast<float2 *>(rec + RC::H2) = make_float2(h[2], l[2]);
             }
         }
-        int li[NPE];
 #pragma unroll
-        for (int i = 0; i < NPE; ++i) li[i] = (int)bounds_clamp(mlidx[i * 32 + lane], U, p.status);
+        for (int i = 0; i < NPE; ++i) li[i] = (int)bounds_clamp(LANECOL ? li[i] : mlidx[i * 32 + lane], U, p.status);
         const bool valid = e >= 0;
         Mat<R> m = p.mat0;
         if (p.mats) m = p.mats[bounds_clamp(p.emat[(size_t)t * 32 + lane], p.n_mats, p.status)];
@@ -496,9 +576,7 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
         if constexpr (MAT == MAT_SVK || MAT == MAT_SVK_KV) m.model = MODEL_SVK;
         const bool visc = MAT == MAT_ANY ? (need_ud && (m.mu_v != R(0) || m.lam_v != R(0)))
                                          : (MAT == MAT_NH_KV || MAT == MAT_SVK_KV);
-        // affine path: J^{-1} and det J of this lane's element (Sec. 6, affine case)
-        R Ji[9], detJ = R(0);
-        if constexpr (AFF) {
+        if constexpr (AFF && !LANECOL) {
             const R *A = reinterpret_cast<const R *>(M + MB) + lane;
 #pragma unroll
             for (int r = 0; r < 9; ++r) Ji[r] = A[r * 32];
@@ -517,7 +595,9 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
         // + (l_i - l_0) as (h_i + (-h_0)) + (l_i + (-l_0)), the same roundings
         float2 nh01 = make_float2(0.f, 0.f), nl01 = make_float2(0.f, 0.f), dp[NPE];
         float nh2 = 0.f, nl2 = 0.f;
-        if constexpr (PK) {
+        if constexpr (LANECOL) {
+            // formed where the nodes are read, below
+        } else if constexpr (PK) {
             const float4 A = lds4(work + li[0] * REC), B = lds4(work + li[0] * REC + 4);
             nh01 = make_float2(-A.x, -A.y);
             nl01 = make_float2(-A.z, -A.w);
@@ -526,7 +606,7 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
         } else {
             ld_u(work + li[0] * REC, h0v, l0v);
         }
-        if constexpr (DD_REG) {
+        if constexpr (DD_REG && !LANECOL) {
 #pragma unroll
             for (int i = 1; i < NPE; ++i) {
                 if constexpr (PK) {
@@ -563,6 +643,11 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
         }
         R gmu_acc = R(0), glam_acc = R(0);
         int bad = 0;
+        int sp[NPE];  // column paths: slot positions, loaded ahead of their use
+        auto load_positions = [&]() {
+#pragma unroll
+            for (int i = 0; i < NPE; ++i) sp[i] = ldg_u16_volatile(spos + i * 32 + lane);
+        };
 
         // ---- the next tile's nodal inputs towards L2 (its metadata was
         // requested at the start of this tile); false when that metadata never
@@ -574,6 +659,17 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
         // without it than with it early or late, also with the L2 flushed
         // before the launch. (The tile-start wait on the metadata barrier
         // stands without it.)
+        // the next tile's per-lane tables towards L2 (column paths): the
+        // 128-byte lines of its local indices and positions, and of its affine record
+        auto prefetch_tables = [&]() {
+            if constexpr (LANECOL) {
+                if (k + 1 >= n_my) return;
+                constexpr int NL = (meta_lane_bytes(NPE) + 127) / 128 + 1, NA = (int)(AffRec<R>::BYTES / 128);
+                const size_t tn = (size_t)(t + tstep);
+                if (lane < NL) prefetch_l2(p.meta + tn * MB + HB + min(lane * 128, meta_lane_bytes(NPE) - 1));
+                else if (lane < NL + NA) prefetch_l2(reinterpret_cast<const unsigned char *>(p.aff + tn * AFF_ROWS * 32) + (lane - NL) * 128);
+            }
+        };
         auto prefetch_next = [&]() -> bool {
             if (k + 1 >= n_my) return true;
             const bool ok = mbar_wait_bounded(mbar + ((k + 1) & 1), (uint32_t)(((k + 1) >> 1) & 1));
@@ -587,11 +683,255 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
                 if (need_ud) prefetch_l2(p.ud + 3 * n);
                 if (HAS_V) prefetch_l2(p.v + 3 * n);
             }
+            prefetch_tables();
             return true;
         };
 
+        // ---- FP32 affine T10 and H8: the fields of the lane's element in its
+        // own shared column, the points two at a time (and the centroid of the
+        // T10 rule alone), the element vectors from the points' operators
+        // (k_t10.cuh, k_h8.cuh)
+        if constexpr (LANECOL) {
+            constexpr int NF = t10_fields(OP, MAT);  // fields held: u, [udot,] [the direction]
+            constexpr int FV = NF - 1;
+            constexpr bool DAMPED = mat_damped(MAT);
+            float *Aj = work + lane;          // the lane's J^{-1}, read again where it is used
+            float *const cols = Aj + 9 * 32;  // the lane's columns
+            // nodal values: displacements relative to node 0 (pair by pair),
+            // velocities, the direction. The columns go over the patch: every
+            // lane reads all of its nodes first
+            auto nodal = [&](V3f(*x)[NPE]) {
+                float4 A0 = make_float4(0.f, 0.f, 0.f, 0.f), B0 = A0;
+#pragma unroll
+                for (int i = 0; i < NPE; ++i) {
+                    const float *rc = work + li[i] * REC;
+                    const float4 A = lds4(rc), B = lds4(rc + 4);
+                    if (i == 0) {
+                        A0 = A;
+                        B0 = B;
+                        x[0][0] = {make_float2(0.f, 0.f), 0.f};
+                    } else {
+                        x[0][i] = {add2(add2(make_float2(A.x, A.y), make_float2(-A0.x, -A0.y)),
+                                        add2(make_float2(A.z, A.w), make_float2(-A0.z, -A0.w))),
+                                   (B.x - B0.x) + (B.y - B0.y)};
+                    }
+                    if constexpr (NF > 1) {
+                        const float4 C4 = lds4(rc + 8);
+                        if constexpr (DAMPED) x[1][i] = {make_float2(C4.x, C4.y), B.z};
+                        if constexpr (HAS_V) x[FV][i] = {make_float2(C4.z, C4.w), B.w};
+                    }
+                }
+                if constexpr (DAMPED)
+                    if (!need_ud)  // the generic law without a velocity: its slots hold nothing
+#pragma unroll
+                        for (int i = 0; i < NPE; ++i) x[1][i] = {make_float2(0.f, 0.f), 0.f};
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < 9; ++r) Aj[r * 32] = Ji[r];
+            };
+            // state and operators of one point or two (V), from the gradients g
+            // of the fields (9 each)
+            auto point = [&](auto *g, auto *T0, auto *T1, R w) {
+                using V = typename std::remove_pointer<decltype(g)>::type;
+                QP<V> s1;
+                V D[9];
+#pragma unroll
+                for (int k2 = 0; k2 < 9; ++k2) {
+                    s1.G[k2] = g[k2];
+                    s1.Fd[k2] = DAMPED ? g[9 + k2] : V(0.f);
+                    D[k2] = HAS_V ? g[FV * 9 + k2] : V(0.f);
+                }
+                stress_state<R>(m, s1, visc);
+                if constexpr (OP == OP_FORCE || OP == OP_FM) first_piola(s1, visc, T0);
+                if constexpr (OP == OP_MATVEC) dstress<R>(m, s1, visc, D, p.aK, p.aC, p.sym_only != 0, T0);
+                if constexpr (OP == OP_FM) dstress<R>(m, s1, visc, D, p.aK, p.aC, false, T1);
+                if constexpr (OP == OP_VJP) {
+                    V gmu, glam;
+                    astress<R>(m, s1, visc, D, T0, T1, gmu, glam);
+                    gmu_acc += w * sum_of(gmu);
+                    glam_acc += w * sum_of(glam);
+                }
+                bad += valid ? count_not(s1.ok) : 0;
+            };
+            auto store = [&](int fo, const V3f *F) {
+#pragma unroll
+                for (int i = 0; i < NPE; ++i) {
+                    (fo == 0 ? ap0 : ap1)[i] = F[i].xy;
+                    (fo == 0 ? acc0 : acc1)[i][2] = F[i].z;
+                }
+            };
+            if constexpr (T10R) {
+            constexpr int NV = 9 * NF;
+            float2 *rec = reinterpret_cast<float2 *>(work + 9 * 32) + lane;
+            float *stash = cols + 4 * NV * 32;  // the lane's mass vector
+            if (!mass_only) {
+                float g0[NV];
+                {
+                    V3f x[NF][NPE];
+                    nodal(x);
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) t10_gradients<NQ, NV>(x[f], Ji, rec + f * 9 * 32, g0 + f * 9);
+                    if constexpr (HAS_V)
+                        if (p.aM != R(0)) {
+                            V3f y[NPE];
+                            t10_mass(x[FV], p.aM * m.rho * p.evol[(size_t)t * 32 + lane], y);
+#pragma unroll
+                            for (int i = 0; i < NPE; ++i) {
+                                stash[(i * 3) * 32] = y[i].xy.x;
+                                stash[(i * 3 + 1) * 32] = y[i].xy.y;
+                                stash[(i * 3 + 2) * 32] = y[i].z;
+                            }
+                        }
+                }
+                if constexpr (PF_NONE) prefetch_tables();
+                if (PF_EARLY && !prefetch_next()) {
+                    timed_out = true;
+                    break;
+                }
+                constexpr float w1 = float(T10Rule<NQ>::w), w0 = float(T10Rule<NQ>::w0);
+                float c0[TWO ? 18 : 9];  // the centroid's operators in units of the other points' weight
+#pragma unroll
+                for (int k2 = 0; k2 < (TWO ? 18 : 9); ++k2) c0[k2] = 0.f;
+                if constexpr (NQ == 5) {
+                    float T0[9], T1[9];
+                    point(g0, T0, T1, w0 * detJ);
+                    constexpr float c = float(T10Rule<NQ>::w0 / (4.0 * T10Rule<NQ>::w));
+#pragma unroll
+                    for (int k2 = 0; k2 < 9; ++k2) {
+                        c0[k2] = c * T0[k2];
+                        if constexpr (TWO) c0[9 + k2] = c * T1[k2];
+                    }
+                }
 #pragma unroll 1
-        for (int q = 0; q < (mass_only ? 0 : NQ); ++q) {
+                for (int h = 0; h < 2; ++h) {
+                    float2 *rh = rec + h * NV * 32;
+                    F2 g[NV], T0[9], T1[9];
+#pragma unroll
+                    for (int k2 = 0; k2 < NV; ++k2) g[k2] = rh[k2 * 32];
+                    point(g, T0, T1, w1 * detJ);
+#pragma unroll
+                    for (int k2 = 0; k2 < 9; ++k2) {
+                        rh[k2 * 32] = NQ == 5 ? add2(T0[k2].v, bc2(c0[k2])) : T0[k2].v;
+                        if constexpr (TWO) rh[(9 + k2) * 32] = NQ == 5 ? add2(T1[k2].v, bc2(c0[9 + k2])) : T1[k2].v;
+                    }
+                }
+                load_positions();
+                float Jw[9];
+#pragma unroll
+                for (int r = 0; r < 9; ++r) Jw[r] = (w1 * detJ) * Aj[r * 32];
+#pragma unroll
+                for (int fo = 0; fo < NFO; ++fo) {
+                    V3f F[NPE];
+                    t10_vectors<NQ, NV>(rec + fo * 9 * 32, Jw, F);
+                    store(fo, F);
+                }
+            }
+            // the mass vector of the lane's element into the operator product
+            // (the second element vector of OP_FM): stashed before the points,
+            // or formed here from the patch where there are none
+            if constexpr (OP == OP_MATVEC || OP == OP_FM)
+                if (p.aM != R(0)) {
+                    float2 *apy = OP == OP_FM ? ap1 : ap0;
+                    R(*accy)[3] = OP == OP_FM ? acc1 : acc0;
+                    if (mass_only) {
+                        load_positions();
+                        V3f xv[NPE], y[NPE];
+#pragma unroll
+                        for (int i = 0; i < NPE; ++i) {
+                            const float *rc = work + li[i] * REC;
+                            xv[i] = {*reinterpret_cast<const float2 *>(rc + RC::V01), rc[RC::V2]};
+                        }
+                        t10_mass(xv, p.aM * m.rho * p.evol[(size_t)t * 32 + lane], y);
+#pragma unroll
+                        for (int i = 0; i < NPE; ++i) {
+                            apy[i] = y[i].xy;
+                            accy[i][2] = y[i].z;
+                        }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < NPE; ++i) {
+                            apy[i] = add2(apy[i], make_float2(stash[(i * 3) * 32], stash[(i * 3 + 1) * 32]));
+                            accy[i][2] += stash[(i * 3 + 2) * 32];
+                        }
+                    }
+                }
+            }
+            if constexpr (H8C) {
+                float *col = cols;  // [NF][7][3] coefficients, then the direction's sum
+                float *vsum = col + 21 * NF * 32;
+                {
+                    V3f x[NF][NPE];
+                    nodal(x);
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) {
+                        h8_transform(x[f]);
+#pragma unroll
+                        for (int c = 1; c < 8; ++c) {
+                            const V3f v = x[f][c] * h8_scale(c);
+                            float *o = col + (f * 21 + (c - 1) * 3) * 32;
+                            o[0] = v.xy.x;
+                            o[32] = v.xy.y;
+                            o[64] = v.z;
+                        }
+                    }
+                    if constexpr (HAS_V) {
+                        vsum[0] = x[FV][0].xy.x;
+                        vsum[32] = x[FV][0].xy.y;
+                        vsum[64] = x[FV][0].z;
+                    }
+                }
+                if constexpr (PF_NONE) prefetch_tables();
+                if (PF_EARLY && !mass_only && !prefetch_next()) {
+                    timed_out = true;
+                    break;
+                }
+                V3f C[NFO][8];
+#pragma unroll
+                for (int fo = 0; fo < NFO; ++fo)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) C[fo][c] = {make_float2(0.f, 0.f), 0.f};
+                constexpr bool PAIR = h8_pairs(OP, MAT);
+                using V = typename std::conditional<PAIR, F2, float>::type;
+#pragma unroll 1
+                for (int q = 0; q < (mass_only ? 0 : (PAIR ? 4 : 8)); ++q) {
+                    const float sy = (q & 1) ? 1.f : -1.f, sz = (q & 2) ? 1.f : -1.f;
+                    V sx, g[9 * NF], T0[9], T1[9];
+                    if constexpr (PAIR) sx = F2(make_float2(-1.f, 1.f));
+                    else sx = (q & 4) ? 1.f : -1.f;
+                    {
+                        float J[9];
+#pragma unroll
+                        for (int r = 0; r < 9; ++r) J[r] = Aj[r * 32];
+#pragma unroll
+                        for (int f = 0; f < NF; ++f) h8_gradients<V>(col + f * 21 * 32, sx, sy, sz, J, g + f * 9);
+                    }
+                    point(g, T0, T1, detJ);
+                    h8_accumulate<V>(T0, sx, sy, sz, Aj, detJ, C[0]);
+                    if constexpr (TWO) h8_accumulate<V>(T1, sx, sy, sz, Aj, detJ, C[1]);
+                }
+                load_positions();
+#pragma unroll
+                for (int fo = 0; fo < NFO; ++fo) {
+#pragma unroll
+                    for (int c = 1; c < 8; ++c) C[fo][c] = C[fo][c] * h8_scale(c);
+                    if constexpr (OP == OP_MATVEC || OP == OP_FM)
+                        if (fo == NFO - 1 && p.aM != R(0)) {
+                            const float r = p.aM * m.rho * p.evol[(size_t)t * 32 + lane];
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) {
+                                const float *o = c == 0 ? vsum : col + (FV * 21 + (c - 1) * 3) * 32;
+                                const float s = r * float(c == 0 ? h8_mass(0) : h8_mass(c) / h8_scale(c));
+                                C[fo][c] = C[fo][c].fma(s, V3f{make_float2(o[0], o[32]), o[64]});
+                            }
+                        }
+                    h8_transform_t(C[fo]);
+                    store(fo, C[fo]);
+                }
+            }
+        }
+
+#pragma unroll 1
+        for (int q = 0; q < (LANECOL || mass_only ? 0 : NQ); ++q) {
             // reference gradients of this point: the slab slice (isoparametric
             // path), or the parent gradients g_i with h_i = J^{-T} g_i (affine path)
             const R *sl = nullptr;
@@ -969,7 +1309,7 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
 
         // consistent mass of affine elements: m_ij = rho V Mhat_ij (Sec. 4.1),
         // into the operator product (the second element vector of OP_FM)
-        if ((OP == OP_MATVEC || OP == OP_DIAG || OP == OP_FM) && p.aM != R(0)) {
+        if (!LANECOL && (OP == OP_MATVEC || OP == OP_DIAG || OP == OP_FM) && p.aM != R(0)) {
             const R c = p.aM * m.rho * p.evol[(size_t)t * 32 + lane];
             if (OP == OP_MATVEC || OP == OP_FM) {
                 float2 *apy = OP == OP_FM ? ap1 : ap0;
@@ -1035,7 +1375,7 @@ __device__ __forceinline__ bool elem_tiles(const KParams<R> &p, unsigned char *w
             if (valid) {
 #pragma unroll
                 for (int i = 0; i < NPE; ++i) {
-                    const int ps = (int)bounds_clamp(spos[i * 32 + lane], NPE * 32, p.status);
+                    const int ps = (int)bounds_clamp(LANECOL ? sp[i] : spos[i * 32 + lane], NPE * 32, p.status);
                     sA[ps] = make_float4(ap0[i].x, ap0[i].y, acc0[i][2], TWO ? ap1[i].x : 0.f);
                     if constexpr (TWO) sB[ps] = make_float2(ap1[i].y, acc1[i][2]);
                 }
@@ -1200,7 +1540,7 @@ __global__ void __launch_bounds__(128, min_ctas<ET, R, OP, AFF, MAT>()) k_elem(c
     const int wib = threadIdx.x >> 5;
     const int wpb = blockDim.x >> 5;
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem) + wib * (NSLICE + 2);  // [wpb][NSLICE + 2] (<= 128 B)
-    unsigned char *wbase = smem + 128 + (size_t)wib * warp_region_bytes<ET, R, OP, AFF>(p.umax, p.meta_bytes);
+    unsigned char *wbase = smem + 128 + (size_t)wib * p.wreg;
 
     const int gw = blockIdx.x * wpb + wib;
     const int W = gridDim.x * wpb;
@@ -1233,8 +1573,10 @@ template <int OP, typename R, bool AFF, int MAT> static void (*kernel_for_(int e
         if (sizeof(R) != 4 || et == ET_Q27) return nullptr;
     }
     if (et == ET_T4 && nq == 1) return k_elem<ET_T4, 1, R, OP, AFF, MAT>;
-    if (et == ET_T10 && nq == 4) return k_elem<ET_T10, 4, R, OP, AFF, MAT>;
-    if (et == ET_T10 && nq == 5) return k_elem<ET_T10, 5, R, OP, AFF, MAT>;
+    if constexpr (!pw_path(ET_T10, AFF, OP, sizeof(R) == 4)) {
+        if (et == ET_T10 && nq == 4) return k_elem<ET_T10, 4, R, OP, AFF, MAT>;
+        if (et == ET_T10 && nq == 5) return k_elem<ET_T10, 5, R, OP, AFF, MAT>;
+    }
     if (et == ET_H8 && nq == 8) return k_elem<ET_H8, 8, R, OP, AFF, MAT>;
     if constexpr (OP != OP_FM)
         if (et == ET_Q27 && nq == 27) return k_elem<ET_Q27, 27, R, OP, AFF, MAT>;
@@ -1267,26 +1609,34 @@ template <int OP, typename R> static void (*kernel_for(int et, int nq, bool aff,
     else return aff ? kernel_for_m<OP, R, true>(et, nq, mat) : kernel_for_m<OP, R, false>(et, nq, mat);
 }
 
-template <int OP, typename R, bool AFF> size_t smem_for_(int et, int umax, int meta_bytes, int wpb)
+// bytes of one warp's shared-memory region in the tile kernels (0: no such kernel)
+template <int OP, typename R, bool AFF> size_t region_for_(int et, int umax, int meta_bytes, int mat, bool mass)
 {
-    if (et == ET_T4) return elem_smem_bytes<ET_T4, R, OP, AFF>(umax, meta_bytes, wpb);
-    if (et == ET_T10) return elem_smem_bytes<ET_T10, R, OP, AFF>(umax, meta_bytes, wpb);
-    if (et == ET_H8) return elem_smem_bytes<ET_H8, R, OP, AFF>(umax, meta_bytes, wpb);
-    if (et == ET_Q27 && OP != OP_FM) return elem_smem_bytes<ET_Q27, R, OP, AFF>(umax, meta_bytes, wpb);
+    if (et == ET_T4) return warp_region_bytes<ET_T4, R, OP, AFF>(umax, meta_bytes, mat, mass);
+    if (et == ET_T10) return warp_region_bytes<ET_T10, R, OP, AFF>(umax, meta_bytes, mat, mass);
+    if (et == ET_H8) return warp_region_bytes<ET_H8, R, OP, AFF>(umax, meta_bytes, mat, mass);
+    if (et == ET_Q27 && OP != OP_FM) return warp_region_bytes<ET_Q27, R, OP, AFF>(umax, meta_bytes, mat, mass);
     return 0;
 }
-template <int OP, typename R> size_t smem_for(int et, int nq, int umax, int meta_bytes, int wpb, bool aff)
+template <int OP, typename R> size_t region_for(int et, int umax, int meta_bytes, bool aff, int mat, bool mass)
+{
+    return aff ? region_for_<OP, R, true>(et, umax, meta_bytes, mat, mass)
+               : region_for_<OP, R, false>(et, umax, meta_bytes, mat, mass);
+}
+template <int OP, typename R>
+size_t smem_for(int et, int nq, int umax, int meta_bytes, int wpb, bool aff, int mat, bool mass)
 {
     if (wpe_path(et, aff)) return OP == OP_FM ? 0 : wpe_smem_bytes<R>(wpb);
     if (pw_path(et, aff, OP, sizeof(R) == 4)) return pw_smem_for<OP>(nq, umax, meta_bytes);
-    return aff ? smem_for_<OP, R, true>(et, umax, meta_bytes, wpb) : smem_for_<OP, R, false>(et, umax, meta_bytes, wpb);
+    const size_t w = region_for<OP, R>(et, umax, meta_bytes, aff, mat, mass);
+    return w ? cta_smem_bytes(w, wpb) : 0;
 }
 
 // resident warps per SM for the best CTA size among 4, 2 and 1 warps, or for
 // the CTA size *wpb_io when it is positive on entry. The point-per-warp
 // kernels have one CTA size, nq warps, which answers for 4.
 template <int OP, typename R>
-int occupancy_op(int et, int nq, bool aff, int mat, int umax, int meta_bytes, int *wpb_io, std::string *why)
+int occupancy_op(int et, int nq, bool aff, int mat, bool mass, int umax, int meta_bytes, int *wpb_io, std::string *why)
 {
     void (*kern)(const KParams<R>) = kernel_for<OP, R>(et, nq, aff, mat);
     const int only = *wpb_io;
@@ -1301,7 +1651,7 @@ int occupancy_op(int et, int nq, bool aff, int mat, int umax, int meta_bytes, in
         if (only > 0 && size != only && !(pw && only == nq)) continue;
         if (pw && size != 4) continue;
         const int wpb = pw ? nq : size;
-        const size_t smem = smem_for<OP, R>(et, nq, umax, meta_bytes, wpb, aff);
+        const size_t smem = smem_for<OP, R>(et, nq, umax, meta_bytes, wpb, aff, mat, mass);
         if (smem > 227 * 1024) continue;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int nb = 0;
@@ -1324,12 +1674,15 @@ int occupancy_op(int et, int nq, bool aff, int mat, int umax, int meta_bytes, in
 // launch on the affine path when p.aff is set, else on the isoparametric
 // (slab) path; material mode p.mat_mode
 template <int OP, typename R>
-cudaError_t launch_op(int et, int nq, const KParams<R> &p, int grid, int wpb, cudaStream_t s)
+cudaError_t launch_op(int et, int nq, const KParams<R> &p0, int grid, int wpb, cudaStream_t s)
 {
+    KParams<R> p = p0;
     const bool aff = p.aff != nullptr;
     void (*kern)(const KParams<R>) = kernel_for<OP, R>(et, nq, aff, p.mat_mode);
     if (!kern) return cudaErrorInvalidValue;
-    const size_t smem = smem_for<OP, R>(et, nq, p.umax, p.meta_bytes, wpb, aff);
+    const bool mass = p.aM != R(0);
+    const size_t smem = smem_for<OP, R>(et, nq, p.umax, p.meta_bytes, wpb, aff, p.mat_mode, mass);
+    p.wreg = (int)region_for<OP, R>(et, p.umax, p.meta_bytes, aff, p.mat_mode, mass);
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     kern<<<grid, 32 * wpb, smem, s>>>(p);

@@ -5,6 +5,6 @@
 namespace tlfe {
 template cudaError_t launch_op<OP_FM, float>(int, int, const KParams<float> &, int, int, cudaStream_t);
 template cudaError_t launch_op<OP_FM, double>(int, int, const KParams<double> &, int, int, cudaStream_t);
-template int occupancy_op<OP_FM, double>(int, int, bool, int, int, int, int *, std::string *);
-template int occupancy_op<OP_FM, float>(int, int, bool, int, int, int, int *, std::string *);
+template int occupancy_op<OP_FM, double>(int, int, bool, int, bool, int, int, int *, std::string *);
+template int occupancy_op<OP_FM, float>(int, int, bool, int, bool, int, int, int *, std::string *);
 }  // namespace tlfe

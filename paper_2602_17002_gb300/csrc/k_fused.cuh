@@ -113,14 +113,15 @@ __global__ void __launch_bounds__(128, fused_min_ctas<OP>()) k_fused(const __gri
     }
 }
 
-// shared-memory region of one warp for a pass of code `code` (affine path)
-template <typename R, int OP> size_t fused_warp_region(int code, int umax, int meta_bytes)
+// shared-memory region of one warp for a pass of code `code` and material
+// mode `mat` (affine path), with room for a mass term
+template <typename R, int OP> size_t fused_warp_region(int code, int umax, int meta_bytes, int mat)
 {
     switch (code) {
-    case FK_T4Q1: return warp_region_bytes<ET_T4, R, OP, true>(umax, meta_bytes);
+    case FK_T4Q1: return warp_region_bytes<ET_T4, R, OP, true>(umax, meta_bytes, mat, true);
     case FK_T10Q4:
-    case FK_T10Q5: return warp_region_bytes<ET_T10, R, OP, true>(umax, meta_bytes);
-    case FK_H8Q8: return warp_region_bytes<ET_H8, R, OP, true>(umax, meta_bytes);
+    case FK_T10Q5: return warp_region_bytes<ET_T10, R, OP, true>(umax, meta_bytes, mat, true);
+    case FK_H8Q8: return warp_region_bytes<ET_H8, R, OP, true>(umax, meta_bytes, mat, true);
     default: return 0;
     }
 }

@@ -3,7 +3,7 @@
 #include "k_fused.cuh"
 
 namespace tlfe {
-template size_t fused_warp_region<float, OP_MATVEC>(int, int, int);
+template size_t fused_warp_region<float, OP_MATVEC>(int, int, int, int);
 template int occupancy_fused<OP_MATVEC, float>(size_t, int *);
 template cudaError_t launch_fused<OP_MATVEC, float>(const FusedArgs<float> &, int, int, cudaStream_t);
 }  // namespace tlfe

@@ -32,7 +32,7 @@ template <typename R> struct FusedArgs {
 
 // defined in k_fused.cuh, instantiated for (OP_FORCE, float) in
 // k_fused_force.cu and (OP_MATVEC, float) in k_fused_matvec.cu
-template <typename R, int OP> size_t fused_warp_region(int code, int umax, int meta_bytes);
+template <typename R, int OP> size_t fused_warp_region(int code, int umax, int meta_bytes, int mat);
 template <int OP, typename R> int occupancy_fused(size_t wreg, int *wpb_io);
 template <int OP, typename R> cudaError_t launch_fused(const FusedArgs<R> &a, int grid, int wpb, cudaStream_t s);
 

@@ -55,6 +55,7 @@ template <typename R> struct KParams {
     //   u16 node offsets[U + 1] into that order (padded)
     const unsigned char *meta;
     int meta_bytes, umaxp;
+    int wreg;                   // bytes of one warp's shared-memory region (set by launch_op)
     const int32_t *eid;         // [n_tiles][32] global element id, -1 for padding lanes
     const int32_t *conn;        // [n_elem][npe] global node ids, block element order (warp-per-element path)
     int elem_base;              // global id of the block's first element
@@ -129,9 +130,11 @@ cudaError_t launch_op(int et, int nq, const KParams<R> &p, int grid, int wpb, cu
 
 // warps per SM the kernel of (op, et, nq, precision, path) can keep resident
 // for a block whose tiles hold at most `umax` unique nodes
-// (CTA sizes of 1, 2 and 4 warps are tried; *wpb receives the best one)
+// (CTA sizes of 1, 2 and 4 warps are tried; *wpb receives the best one);
+// mass: the operation has a mass term (a_M != 0), which takes shared memory
+// on the T10 path
 template <int OP, typename R>
-int occupancy_op(int et, int nq, bool aff, int mat, int umax, int meta_bytes, int *wpb, std::string *why);
+int occupancy_op(int et, int nq, bool aff, int mat, bool mass, int umax, int meta_bytes, int *wpb, std::string *why);
 
 // set-up kernels
 cudaError_t launch_precompute(int et, int nq, int precision, int n_tiles, const int32_t *eid,

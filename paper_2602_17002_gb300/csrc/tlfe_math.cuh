@@ -60,6 +60,68 @@ template <typename R> struct Mat {
 };
 
 // ---------------------------------------------------------------------------
+// Two quadrature points of one element in one FP32x2 register pair: every
+// operation below is one packed instruction for both (negated, swapped and
+// broadcast operands cost nothing). A product is kept open until it is used,
+// so that sums of products become packed multiply-adds, as the compiler makes
+// them of the scalar types.
+// ---------------------------------------------------------------------------
+struct F2 {
+    float2 v;
+    __device__ __forceinline__ F2() {}
+    __device__ __forceinline__ F2(float x) : v(make_float2(x, x)) {}
+    __device__ __forceinline__ F2(float2 x) : v(x) {}
+};
+struct F2Prod {
+    float2 a, b;
+    __device__ __forceinline__ operator F2() const { return __fmul2_rn(a, b); }
+};
+__device__ __forceinline__ float2 neg2(float2 x) { return make_float2(-x.x, -x.y); }
+__device__ __forceinline__ F2 operator-(F2 x) { return neg2(x.v); }
+__device__ __forceinline__ F2Prod operator-(F2Prod p) { return {neg2(p.a), p.b}; }
+__device__ __forceinline__ F2Prod operator*(F2 a, F2 b) { return {a.v, b.v}; }
+__device__ __forceinline__ F2Prod operator*(F2 a, float b) { return {a.v, make_float2(b, b)}; }
+__device__ __forceinline__ F2Prod operator*(float a, F2 b) { return {make_float2(a, a), b.v}; }
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) { return __fadd2_rn(a.v, b.v); }
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return __fadd2_rn(a.v, neg2(b.v)); }
+__device__ __forceinline__ F2 operator+(F2Prod p, F2 c) { return __ffma2_rn(p.a, p.b, c.v); }
+__device__ __forceinline__ F2 operator+(F2 c, F2Prod p) { return __ffma2_rn(p.a, p.b, c.v); }
+__device__ __forceinline__ F2 operator+(F2Prod p, F2Prod q) { return __ffma2_rn(q.a, q.b, __fmul2_rn(p.a, p.b)); }
+__device__ __forceinline__ F2 operator-(F2Prod p, F2 c) { return __ffma2_rn(p.a, p.b, neg2(c.v)); }
+__device__ __forceinline__ F2 operator-(F2 c, F2Prod p) { return __ffma2_rn(neg2(p.a), p.b, c.v); }
+__device__ __forceinline__ F2 operator-(F2Prod p, F2Prod q) { return __ffma2_rn(neg2(q.a), q.b, __fmul2_rn(p.a, p.b)); }
+template <typename T> __device__ __forceinline__ F2 &operator+=(F2 &a, const T &b) { return a = a + b; }
+
+// the scalar type of a value type, and per-point truth values
+template <typename V> struct ValueOf {
+    using S = V;
+    using Mask = bool;
+};
+struct Mask2 {
+    bool x, y;
+};
+template <> struct ValueOf<F2> {
+    using S = float;
+    using Mask = Mask2;
+};
+__device__ __forceinline__ bool positive(float x) { return x > 0.f; }
+__device__ __forceinline__ bool positive(double x) { return x > 0.0; }
+__device__ __forceinline__ Mask2 positive(F2 x) { return {x.v.x > 0.f, x.v.y > 0.f}; }
+__device__ __forceinline__ bool all_of(bool m) { return m; }
+__device__ __forceinline__ bool all_of(Mask2 m) { return m.x && m.y; }
+__device__ __forceinline__ int count_not(bool m) { return m ? 0 : 1; }
+__device__ __forceinline__ int count_not(Mask2 m) { return (m.x ? 0 : 1) + (m.y ? 0 : 1); }
+template <typename R> __device__ __forceinline__ R where(bool m, R a, R b) { return m ? a : b; }
+__device__ __forceinline__ F2 where(Mask2 m, F2 a, F2 b)
+{
+    return make_float2(m.x ? a.v.x : b.v.x, m.y ? a.v.y : b.v.y);
+}
+__device__ __forceinline__ float sum_of(float x) { return x; }  // over the points of the value
+__device__ __forceinline__ float sum_of(F2 x) { return x.v.x + x.v.y; }
+__device__ __forceinline__ void set_true(bool &m) { m = true; }
+__device__ __forceinline__ void set_true(Mask2 &m) { m.x = m.y = true; }
+
+// ---------------------------------------------------------------------------
 // 3x3 helpers on row-major register arrays
 // ---------------------------------------------------------------------------
 
@@ -96,7 +158,7 @@ __device__ __forceinline__ void mm3(const float A[9], const float B[9], float C[
 // (B, dE of a direction) that are summed with their transpose keep the
 // off-diagonal sums unhalved ("engineering" shear): entry xy of eng(A, B)
 // is (A^T B)_xy + (A^T B)_yx, the diagonal is that of A^T B.
-template <typename R> __device__ __forceinline__ void sym_eng(const R A[9], const R B[9], R e[6])
+template <typename V> __device__ __forceinline__ void sym_eng(const V A[9], const V B[9], V e[6])
 {
 #pragma unroll
     for (int a = 0; a < 3; ++a) e[a] = A[a] * B[a] + A[3 + a] * B[3 + a] + A[6 + a] * B[6 + a];
@@ -106,13 +168,13 @@ template <typename R> __device__ __forceinline__ void sym_eng(const R A[9], cons
 }
 
 // S : e for a symmetric S and an engineering e (the doubled off-diagonals are in e)
-template <typename R> __device__ __forceinline__ R dot6(const R S[6], const R e[6])
+template <typename V> __device__ __forceinline__ V dot6(const V S[6], const V e[6])
 {
     return S[0] * e[0] + S[1] * e[1] + S[2] * e[2] + S[3] * e[3] + S[4] * e[4] + S[5] * e[5];
 }
 
 // cofactors of a symmetric matrix
-template <typename R> __device__ __forceinline__ void cof6(const R B[6], R c[6])
+template <typename V> __device__ __forceinline__ void cof6(const V B[6], V c[6])
 {
     c[0] = B[1] * B[2] - B[5] * B[5];
     c[1] = B[0] * B[2] - B[4] * B[4];
@@ -124,9 +186,9 @@ template <typename R> __device__ __forceinline__ void cof6(const R B[6], R c[6])
 
 // derivative of cof6 at C along dC = 2 sym, given e = eng(F, dF) = (dE_xx, .., 2 dE_xy, ..):
 // diagonal entries halved (d/2), off-diagonal ones whole
-template <typename R> __device__ __forceinline__ void dcof6(const R C[6], const R e[6], R d[6])
+template <typename V> __device__ __forceinline__ void dcof6(const V C[6], const V e[6], V d[6])
 {
-    const R t0 = e[0] + e[0], t1 = e[1] + e[1], t2 = e[2] + e[2];
+    const V t0 = e[0] + e[0], t1 = e[1] + e[1], t2 = e[2] + e[2];
     d[0] = C[1] * e[2] + C[2] * e[1] - C[5] * e[5];
     d[1] = C[0] * e[2] + C[2] * e[0] - C[4] * e[4];
     d[2] = C[0] * e[1] + C[1] * e[0] - C[3] * e[3];
@@ -136,7 +198,7 @@ template <typename R> __device__ __forceinline__ void dcof6(const R C[6], const 
 }
 
 // P = A S with S symmetric (6 entries)
-template <typename R> __device__ __forceinline__ void mm6(const R A[9], const R S[6], R P[9])
+template <typename V> __device__ __forceinline__ void mm6(const V A[9], const V S[6], V P[9])
 {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -145,7 +207,7 @@ template <typename R> __device__ __forceinline__ void mm6(const R A[9], const R 
         P[a * 3 + 2] = A[a * 3] * S[4] + A[a * 3 + 1] * S[5] + A[a * 3 + 2] * S[2];
     }
 }
-template <typename R> __device__ __forceinline__ void mm6_acc(const R A[9], const R S[6], R P[9])
+template <typename V> __device__ __forceinline__ void mm6_acc(const V A[9], const V S[6], V P[9])
 {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -189,43 +251,55 @@ __device__ __forceinline__ void mm6_acc(const float A[9], const float S[6], floa
 // Constitutive state at one quadrature point
 // ---------------------------------------------------------------------------
 
-// Per-point quantities kept between the stress and its derivatives.
-template <typename R> struct QP {
-    R F[9];    // I + G
-    R G[9];    // sum u_i h_i^T
-    R Fd[9];   // sum udot_i h_i^T (valid when visc)
-    R S[6];    // elastic second Piola-Kirchhoff stress
-    R Sv[6];   // viscous second Piola-Kirchhoff stress (valid when visc)
-    R B[6];    // C - I
-    R N[6];    // MR / NH: B - cof(B)
+// Per-point quantities kept between the stress and its derivatives (V: one
+// point, or two of one element in F2).
+template <typename V> struct QP {
+    V F[9];    // I + G
+    V G[9];    // sum u_i h_i^T
+    V Fd[9];   // sum udot_i h_i^T (valid when visc)
+    V S[6];    // elastic second Piola-Kirchhoff stress
+    V Sv[6];   // viscous second Piola-Kirchhoff stress (valid when visc)
+    V B[6];    // C - I
+    V N[6];    // MR / NH: B - cof(B)
     // MR / NH: alpha, alpha s - beta, and the scalars of the header comment
-    R al, c1, s, i, t1;   // t1 = 1 + t
-    R rD, rJ, r1;         // J^{-2}, 1/J, J^{-1/3}
-    R Jm1r;               // (J - 1) / J
-    bool ok;
+    V al, c1, s, i, t1;   // t1 = 1 + t
+    V rD, rJ, r1;         // J^{-2}, 1/J, J^{-1/3}
+    V Jm1r;               // (J - 1) / J
+    typename ValueOf<V>::Mask ok;
 };
 
-template <typename R> __device__ __forceinline__ R rcbrt_(R x);
-template <> __device__ __forceinline__ float rcbrt_<float>(float x) { return rcbrtf(x); }
-template <> __device__ __forceinline__ double rcbrt_<double>(double x) { return rcbrt(x); }
+__device__ __forceinline__ float rcbrt_(float x) { return rcbrtf(x); }
+__device__ __forceinline__ double rcbrt_(double x) { return rcbrt(x); }
+__device__ __forceinline__ F2 rcbrt_(F2 x) { return make_float2(rcbrtf(x.v.x), rcbrtf(x.v.y)); }
+
+// factors of M2 = x1 B - x2 cof(B) + x0 I (see the header comment)
+template <typename R, typename V>
+__device__ __forceinline__ void mr_factors(V t, V I2, V I3, V &x0, V &x1, V &x2)
+{
+    const R third = R(1.0 / 3.0);
+    const V t1 = t + V(R(1));
+    x1 = third * (t - I2) - I3 + V(R(1));
+    x2 = (R(2) * third) * (R(2) * t + I2 + V(R(3)));
+    x0 = (I2 + I3) * (t + V(R(2))) - V(third * t) * t1 - V((R(2) * third) * I2) * t1;
+}
 
 // Elastic and viscous stress state. visc: whether Fd is meaningful and the
-// material damped. Sets q.ok = false (and no elastic part) when the
+// material damped. Clears q.ok (and leaves no elastic part) where the
 // neo-Hookean law meets J <= 0 or a J that is not a number.
-template <typename R> __device__ __forceinline__ void stress_state(const Mat<R> &m, QP<R> &q, bool visc)
+template <typename R, typename V> __device__ __forceinline__ void stress_state(const Mat<R> &m, QP<V> &q, bool visc)
 {
-    const R *G = q.G;
+    const V *G = q.G;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) q.F[k] = G[k] + ((k % 4 == 0) ? R(1) : R(0));
-    q.ok = true;
+    for (int k = 0; k < 9; ++k) q.F[k] = k % 4 == 0 ? G[k] + V(R(1)) : G[k];
+    set_true(q.ok);
     if (visc) {
         // Edot = sym(Fd^T F); S^v = 2 mu_v Edot + lam_v tr(Edot) I  (Sec. 3.2.3)
-        R e[6];
-        sym_eng(q.Fd, q.F, e);
-        const R i = m.lam_v * (e[0] + e[1] + e[2]);
+        V e[6];
+        sym_eng<V>(q.Fd, q.F, e);
+        const V i = m.lam_v * (e[0] + e[1] + e[2]);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            q.Sv[k] = R(2) * m.mu_v * e[k] + i;
+            q.Sv[k] = (R(2) * m.mu_v) * e[k] + i;
             q.Sv[3 + k] = m.mu_v * e[3 + k];
         }
     }
@@ -235,10 +309,10 @@ template <typename R> __device__ __forceinline__ void stress_state(const Mat<R> 
     q.B[3] = G[1] + G[3] + G[0] * G[1] + G[3] * G[4] + G[6] * G[7];
     q.B[4] = G[2] + G[6] + G[0] * G[2] + G[3] * G[5] + G[6] * G[8];
     q.B[5] = G[5] + G[7] + G[1] * G[2] + G[4] * G[5] + G[7] * G[8];
-    const R t = q.B[0] + q.B[1] + q.B[2];
+    const V t = q.B[0] + q.B[1] + q.B[2];
     if (m.model == MODEL_SVK) {
         // S = lam tr(E) I + 2 mu E  (App. C SVK)
-        const R i = R(0.5) * m.lam * t;
+        const V i = (R(0.5) * m.lam) * t;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             q.S[k] = m.mu * q.B[k] + i;
@@ -248,81 +322,92 @@ template <typename R> __device__ __forceinline__ void stress_state(const Mat<R> 
     }
     // neo-Hookean: mu10 = mu/2, k = lam + 2 mu / 3
     const R third = R(1.0 / 3.0);
-    const R c0 = G[4] * G[8] - G[5] * G[7], c1 = G[5] * G[6] - G[3] * G[8], c2 = G[3] * G[7] - G[4] * G[6];
-    const R dG = G[0] * c0 + G[1] * c1 + G[2] * c2;
-    const R I2G = c0 + (G[0] * G[4] - G[1] * G[3]) + (G[0] * G[8] - G[2] * G[6]);
-    const R Jm1 = tr3(G) + I2G + dG;
-    const R J = R(1) + Jm1;
-    if (!(J > R(0))) {
-        q.ok = false;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) q.S[k] = q.N[k] = q.B[k] = R(0);
-        q.al = q.c1 = q.s = q.i = q.t1 = q.rD = q.rJ = q.r1 = q.Jm1r = R(0);
-        return;
-    }
-    const R r = rcbrt_<R>(J), r2 = r * r;
+    const V c0 = G[4] * G[8] - G[5] * G[7], c1 = G[5] * G[6] - G[3] * G[8], c2 = G[3] * G[7] - G[4] * G[6];
+    const V dG = G[0] * c0 + G[1] * c1 + G[2] * c2;
+    const V I2G = c0 + (G[0] * G[4] - G[1] * G[3]) + (G[0] * G[8] - G[2] * G[6]);
+    const V Jm1 = (G[0] + G[4] + G[8]) + I2G + dG;
+    const V J = Jm1 + V(R(1));
+    q.ok = positive(J);
+    const V r = rcbrt_(where(q.ok, J, V(R(1)))), r2 = r * r;
     q.r1 = r;
     q.rJ = r2 * r;
     q.rD = q.rJ * q.rJ;
     q.Jm1r = Jm1 * q.rJ;
-    q.al = (m.mu - R(2) * m.mu01) * (q.rD * r2);
-    const R be = (m.lam + R(2) * third * m.mu) * q.Jm1r;
-    R cB[6];
-    cof6(q.B, cB);
-    const R I2 = cB[0] + cB[1] + cB[2];
-    const R I3 = q.B[0] * cB[0] + q.B[3] * cB[3] + q.B[4] * cB[4];
-    q.t1 = R(1) + t;
-    q.s = R(1) + third * t;
-    q.i = (I2 + I3) - third * t * q.t1;
+    q.al = (m.mu - R(2) * m.mu01) * V(q.rD * r2);
+    const V be = (m.lam + R(2) * third * m.mu) * q.Jm1r;
+    V cB[6];
+    cof6<V>(q.B, cB);
+    const V I2 = cB[0] + cB[1] + cB[2];
+    const V I3 = q.B[0] * cB[0] + q.B[3] * cB[3] + q.B[4] * cB[4];
+    q.t1 = t + V(R(1));
+    q.s = third * t + V(R(1));
+    q.i = (I2 + I3) - V(third * t) * q.t1;
     q.c1 = q.al * q.s - be;
-    const R iso = q.al * q.i + be * q.t1;
+    const V iso = q.al * q.i + be * q.t1;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         q.N[k] = q.B[k] - cB[k];
-        q.S[k] = k < 3 ? q.c1 * q.N[k] + iso : q.c1 * q.N[k];
+        q.S[k] = k < 3 ? V(q.c1 * q.N[k] + iso) : V(q.c1 * q.N[k]);
     }
     if (m.model == MODEL_MR) {
-        const R a2 = R(2) * m.mu01 * q.rD * q.rJ * r;  // 2 mu01 J^{-10/3}
-        const R x1 = R(1) + third * (t - I2) - I3;
-        const R x2 = R(2) * third * (R(3) + R(2) * t + I2);
-        const R x0 = (I2 + I3) * (R(2) + t) - third * t * q.t1 - R(2) * third * I2 * q.t1;
+        const V a2 = (R(2) * m.mu01) * V(V(q.rD * q.rJ) * r);  // 2 mu01 J^{-10/3}
+        V x0, x1, x2;
+        mr_factors<R, V>(t, I2, I3, x0, x1, x2);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const R M2 = x1 * q.B[k] - x2 * cB[k] + (k < 3 ? x0 : R(0));
+            const V M2 = x1 * q.B[k] - x2 * cB[k] + (k < 3 ? x0 : V(R(0)));
             q.S[k] += a2 * M2;
         }
+    }
+    if (!all_of(q.ok)) {
+        const V z = V(R(0));
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            q.S[k] = where(q.ok, q.S[k], z);
+            q.N[k] = where(q.ok, q.N[k], z);
+            q.B[k] = where(q.ok, q.B[k], z);
+        }
+        q.al = where(q.ok, q.al, z);
+        q.c1 = where(q.ok, q.c1, z);
+        q.s = where(q.ok, q.s, z);
+        q.i = where(q.ok, q.i, z);
+        q.t1 = where(q.ok, q.t1, z);
+        q.rD = where(q.ok, q.rD, z);
+        q.Jm1r = where(q.ok, q.Jm1r, z);
     }
 }
 
 // first Piola-Kirchhoff stress of the state: F (S + S^v)
-template <typename R> __device__ __forceinline__ void first_piola(const QP<R> &q, bool visc, R P[9])
+template <typename V> __device__ __forceinline__ void first_piola(const QP<V> &q, bool visc, V P[9])
 {
-    R St[6];
+    using R = typename ValueOf<V>::S;
+    V St[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) St[k] = visc ? q.S[k] + q.Sv[k] : q.S[k];
     mm6(q.F, St, P);
-    if (!q.ok && !visc)  // an F that is not a number leaves no trace
+    if (!all_of(q.ok) && !visc)  // an F that is not a number leaves no trace
 #pragma unroll
-        for (int k = 0; k < 9; ++k) P[k] = R(0);
+        for (int k = 0; k < 9; ++k) P[k] = where(q.ok, P[k], V(R(0)));
 }
 
-template <typename R>
-__device__ __forceinline__ void stress(const Mat<R> &m, QP<R> &q, bool visc, R P[9])
+template <typename R, typename V>
+__device__ __forceinline__ void stress(const Mat<R> &m, QP<V> &q, bool visc, V P[9])
 {
-    stress_state<R>(m, q, visc);
-    first_piola<R>(q, visc, P);
+    stress_state<R, V>(m, q, visc);
+    first_piola<V>(q, visc, P);
 }
 
 // c times the elastic derivative dS along e = eng(F, dF)
-template <typename R>
-__device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<R> &q, const R e[6], R c, R dS[6])
+template <typename R, typename V>
+__device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<V> &q, const V e[6], R c, V dS[6])
 {
-    const R trE = e[0] + e[1] + e[2];
+    const V trE = e[0] + e[1] + e[2];
     if (m.model == MODEL_SVK) {
-        const R i = c * m.lam * trE, a = c * m.mu;
+        const R a = c * m.mu;
+        const V i = (c * m.lam) * trE;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            dS[k] = R(2) * a * e[k] + i;
+            dS[k] = (R(2) * a) * e[k] + i;
             dS[3 + k] = a * e[3 + k];
         }
         return;
@@ -333,48 +418,50 @@ __device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<R> &q, cons
     //   dC^{-1} = (dQ - 2 j Q) / J^2
     const R third = R(1.0 / 3.0);
     const R kb = m.lam + R(2) * third * m.mu;
-    const R as = q.al * q.s;  // alpha I1 / 3; beta = as - c1
-    const R QE = q.t1 * trE - dot6(q.N, e);
-    const R j = QE * q.rD;
-    const R a23 = c * R(2) * third * q.al;
-    const R xM = -a23 * j;
-    const R xQ = c * j * (kb + as + q.c1) - a23 * trE;
-    const R xd = -c * q.c1;
-    const R y1 = xM * q.s - xQ, y0 = xM * q.i + xQ * q.t1;
-    R C[6], dQ[6];
+    const V QE = q.t1 * trE - dot6<V>(q.N, e);
+    const V j = QE * q.rD;
+    const V a23 = (c * R(2) * third) * q.al;
+    const V xM = a23 * -j;
+    const V cj = c * j;
+    // alpha s is alpha I1 / 3; beta = alpha s - c1
+    const V xQ = cj * (q.al * q.s + q.c1 + V(kb)) - a23 * trE;
+    const V xd = -c * q.c1;
+    const V xd2 = xd + xd;
+    const V y1 = xM * q.s - xQ, y0 = xM * q.i + xQ * q.t1;
+    V C[6], dQ[6];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) C[k] = k < 3 ? R(1) + q.B[k] : q.B[k];
-    dcof6(C, e, dQ);
+    for (int k = 0; k < 6; ++k) C[k] = k < 3 ? q.B[k] + V(R(1)) : q.B[k];
+    dcof6<V>(C, e, dQ);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) dS[k] = k < 3 ? y1 * q.N[k] + (R(2) * xd * dQ[k] + y0) : y1 * q.N[k] + xd * dQ[k];
+    for (int k = 0; k < 6; ++k)
+        dS[k] = k < 3 ? V(y1 * q.N[k] + V(xd2 * dQ[k] + y0)) : V(y1 * q.N[k] + xd * dQ[k]);
     if (m.model == MODEL_MR) {
         // S2 = a2 M2, a2 = 2 mu01 J^{-10/3}: dS2 = -(10/3) j S2 + a2 dM2
-        const R t = q.B[0] + q.B[1] + q.B[2];
-        R cB[6];
-        cof6(q.B, cB);
-        const R I2 = cB[0] + cB[1] + cB[2];
-        const R I3 = q.B[0] * cB[0] + q.B[3] * cB[3] + q.B[4] * cB[4];
-        const R x1 = R(1) + third * (t - I2) - I3;
-        const R x2 = R(2) * third * (R(3) + R(2) * t + I2);
-        const R x0 = (I2 + I3) * (R(2) + t) - third * t * (R(1) + t) - R(2) * third * I2 * (R(1) + t);
-        const R a2 = R(2) * m.mu01 * q.rD * q.rJ * q.r1;  // 2 mu01 J^{-10/3}
+        const V t = q.B[0] + q.B[1] + q.B[2];
+        V cB[6];
+        cof6<V>(q.B, cB);
+        const V I2 = cB[0] + cB[1] + cB[2];
+        const V I3 = q.B[0] * cB[0] + q.B[3] * cB[3] + q.B[4] * cB[4];
+        V x0, x1, x2;
+        mr_factors<R, V>(t, I2, I3, x0, x1, x2);
+        const V a2 = (R(2) * m.mu01) * V(V(q.rD * q.rJ) * q.r1);  // 2 mu01 J^{-10/3}
         // invariants of B along dB = 2 dE
-        R dcB[6];
-        dcof6(q.B, e, dcB);  // diagonal halved
-        const R dt = R(2) * trE;
-        const R dI2 = R(2) * (dcB[0] + dcB[1] + dcB[2]);
-        const R dI3 = R(2) * (cB[0] * e[0] + cB[1] * e[1] + cB[2] * e[2] + cB[3] * e[3] + cB[4] * e[4] + cB[5] * e[5]);
-        const R dx1 = third * (dt - dI2) - dI3;
-        const R dx2 = R(2) * third * (R(2) * dt + dI2);
-        const R dx0 = (dI2 + dI3) * (R(2) + t) + (I2 + I3) * dt - third * dt * (R(1) + R(2) * t) -
-                      R(2) * third * (dI2 * (R(1) + t) + I2 * dt);
+        V dcB[6];
+        dcof6<V>(q.B, e, dcB);  // diagonal halved
+        const V dt = R(2) * trE;
+        const V dI2 = R(2) * (dcB[0] + dcB[1] + dcB[2]);
+        const V dI3 = R(2) * dot6<V>(cB, e);
+        const V dx1 = third * (dt - dI2) - dI3;
+        const V dx2 = (R(2) * third) * (R(2) * dt + dI2);
+        const V dx0 = (dI2 + dI3) * (t + V(R(2))) + (I2 + I3) * dt - V(third * dt) * (R(2) * t + V(R(1))) -
+                      V((R(2) * third) * dI2) * (t + V(R(1))) - V((R(2) * third) * I2) * dt;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const R M2 = x1 * q.B[k] - x2 * cB[k] + (k < 3 ? x0 : R(0));
-            const R dB = k < 3 ? R(2) * e[k] : e[k];
-            const R dc = k < 3 ? R(2) * dcB[k] : dcB[k];
-            const R dM2 = dx1 * q.B[k] + x1 * dB - dx2 * cB[k] - x2 * dc + (k < 3 ? dx0 : R(0));
-            dS[k] += c * a2 * (dM2 - R(10) * third * j * M2);
+            const V M2 = x1 * q.B[k] - x2 * cB[k] + (k < 3 ? x0 : V(R(0)));
+            const V dB = k < 3 ? e[k] + e[k] : e[k];
+            const V dc = k < 3 ? dcB[k] + dcB[k] : dcB[k];
+            const V dM2 = dx1 * q.B[k] + x1 * dB - dx2 * cB[k] - x2 * dc + (k < 3 ? dx0 : V(R(0)));
+            dS[k] += V(c * a2) * (dM2 - V((R(10) * third) * j) * M2);
         }
     }
 }
@@ -385,23 +472,24 @@ __device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<R> &q, cons
 // with dF = dFd the given direction; cK scales everything depending on dF, cC
 // everything depending on dFd. sym_only drops the viscous stiffness K^v (the
 // non-symmetric part).
-template <typename R>
-__device__ __forceinline__ void dstress(const Mat<R> &m, const QP<R> &q, bool visc, const R dF[9],
-                                        R cK, R cC, bool sym_only, R dP[9])
+template <typename R, typename V>
+__device__ __forceinline__ void dstress(const Mat<R> &m, const QP<V> &q, bool visc, const V dF[9],
+                                        R cK, R cC, bool sym_only, V dP[9])
 {
-    R e[6], T[6];
-    sym_eng(q.F, dF, e);
+    V e[6], T[6];
+    sym_eng<V>(q.F, dF, e);
     if (cK != R(0)) {
-        R Sk[6];
-        dS_elastic<R>(m, q, e, cK, T);
+        V Sk[6];
+        dS_elastic<R, V>(m, q, e, cK, T);
         const bool vk = visc && !sym_only;
         if (vk) {  // position-side viscous derivative: dEdot = sym(Fd^T dF)
-            R ev[6];
-            sym_eng(q.Fd, dF, ev);
-            const R a = cK * m.mu_v, i = cK * m.lam_v * (ev[0] + ev[1] + ev[2]);
+            V ev[6];
+            sym_eng<V>(q.Fd, dF, ev);
+            const R a = cK * m.mu_v;
+            const V i = (cK * m.lam_v) * (ev[0] + ev[1] + ev[2]);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                T[k] += R(2) * a * ev[k] + i;
+                T[k] += (R(2) * a) * ev[k] + i;
                 T[3 + k] += a * ev[3 + k];
             }
         }
@@ -410,70 +498,71 @@ __device__ __forceinline__ void dstress(const Mat<R> &m, const QP<R> &q, bool vi
         mm6(dF, Sk, dP);
     } else {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) T[k] = R(0);
+        for (int k = 0; k < 6; ++k) T[k] = V(R(0));
 #pragma unroll
-        for (int k = 0; k < 9; ++k) dP[k] = R(0);
+        for (int k = 0; k < 9; ++k) dP[k] = V(R(0));
     }
     if (cC != R(0)) {  // velocity direction: dEdot = sym(F^T dFd)
-        const R a = cC * m.mu_v, i = cC * m.lam_v * (e[0] + e[1] + e[2]);
+        const R a = cC * m.mu_v;
+        const V i = (cC * m.lam_v) * (e[0] + e[1] + e[2]);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            T[k] += R(2) * a * e[k] + i;
+            T[k] += (R(2) * a) * e[k] + i;
             T[3 + k] += a * e[3 + k];
         }
     }
     mm6_acc(q.F, T, dP);
-    if (!q.ok && !(visc && !sym_only) && !(cC != R(0) && (m.mu_v != R(0) || m.lam_v != R(0))))
+    if (!all_of(q.ok) && !(visc && !sym_only) && !(cC != R(0) && (m.mu_v != R(0) || m.lam_v != R(0))))
 #pragma unroll
-        for (int k = 0; k < 9; ++k) dP[k] = R(0);
+        for (int k = 0; k < 9; ++k) dP[k] = where(q.ok, dP[k], V(R(0)));
 }
 
 // Adjoint of the stress map at one point against a cotangent Gh (=sum r_i h_i^T):
 //   gF  = (dP/dF)^T [Gh]  (elastic part self-adjoint; viscous part explicit)
 //   gFd = (dP/dFd)^T [Gh]
 //   gmu = dP/dmu : Gh, glam = dP/dlam : Gh, contracted as dS/dmu : sym(F^T Gh)
-template <typename R>
-__device__ __forceinline__ void astress(const Mat<R> &m, const QP<R> &q, bool visc, const R Gh[9],
-                                        R gF[9], R gFd[9], R &gmu, R &glam)
+template <typename R, typename V>
+__device__ __forceinline__ void astress(const Mat<R> &m, const QP<V> &q, bool visc, const V Gh[9],
+                                        V gF[9], V gFd[9], V &gmu, V &glam)
 {
-    R e[6], T[6], St[6];
-    sym_eng(q.F, Gh, e);
-    dS_elastic<R>(m, q, e, R(1), T);
+    V e[6], T[6], St[6];
+    sym_eng<V>(q.F, Gh, e);
+    dS_elastic<R, V>(m, q, e, R(1), T);
 #pragma unroll
     for (int k = 0; k < 6; ++k) St[k] = visc ? q.S[k] + q.Sv[k] : q.S[k];
     mm6(Gh, St, gF);
     mm6_acc(q.F, T, gF);
-    const R trE = e[0] + e[1] + e[2];
+    const V trE = e[0] + e[1] + e[2];
     if (visc) {
         // L = (F S^v) : Gh, Ebar = 2 mu_v sym(F^T Gh) + lam_v tr I:
         // dL/dF = Gh S^v + Fd Ebar, dL/dFd = F Ebar
-        R Eb[6];
-        const R i = m.lam_v * trE;
+        V Eb[6];
+        const V i = m.lam_v * trE;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            Eb[k] = R(2) * m.mu_v * e[k] + i;
+            Eb[k] = (R(2) * m.mu_v) * e[k] + i;
             Eb[3 + k] = m.mu_v * e[3 + k];
         }
         mm6_acc(q.Fd, Eb, gF);
         mm6(q.F, Eb, gFd);
     } else {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            gFd[k] = R(0);
-            if (!q.ok) gF[k] = R(0);
-        }
+        for (int k = 0; k < 9; ++k) gFd[k] = V(R(0));
+        if (!all_of(q.ok))
+#pragma unroll
+            for (int k = 0; k < 9; ++k) gF[k] = where(q.ok, gF[k], V(R(0)));
     }
     if (m.model == MODEL_SVK) {
         // dS/dlam = tr(E) I, dS/dmu = 2 E = B
-        gmu = dot6(q.B, e);
-        glam = R(0.5) * (q.B[0] + q.B[1] + q.B[2]) * trE;
+        gmu = dot6<V>(q.B, e);
+        glam = V(R(0.5) * (q.B[0] + q.B[1] + q.B[2])) * trE;
     } else {
         // dS/dmu = J^{-8/3} M + 2/3 (J - 1)/J Q (mu01 held fixed), dS/dlam = (J - 1)/J Q
-        const R NE = dot6(q.N, e);
-        const R gq = q.Jm1r * (q.t1 * trE - NE);
-        const R g = q.rD * q.r1 * q.r1 * (q.s * NE + q.i * trE) + R(2.0 / 3.0) * gq;
-        gmu = q.ok ? g : R(0);
-        glam = q.ok ? gq : R(0);
+        const V NE = dot6<V>(q.N, e);
+        const V gq = q.Jm1r * (q.t1 * trE - NE);
+        const V g = V(V(q.rD * q.r1) * q.r1) * (q.s * NE + q.i * trE) + R(2.0 / 3.0) * gq;
+        gmu = where(q.ok, g, V(R(0)));
+        glam = where(q.ok, gq, V(R(0)));
     }
 }
 

@@ -20,6 +20,7 @@ struct NewtonState;  // newton.cu
 // One element block as stored on the device.
 struct LaunchSched {
     int resident = 0;   // resident warps per SM at wpb warps per CTA (0: not resident)
+    int resident_mass = 0;  // the same with a mass term (0: not asked for yet)
     int wpb = 0;        // warps per CTA
     int chunk = 0;      // 1: contiguous tile runs per warp; 0: interleaved
     bool tuned = false; // chosen by measurement
