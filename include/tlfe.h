@@ -103,11 +103,11 @@ enum { TLFE_PATH_AUTO = 0, TLFE_PATH_SLAB = 1, TLFE_PATH_AFFINE = 2 };
 enum { TLFE_PATCH_BANKED = 0, TLFE_PATCH_SORTED = 1 };
 /* How the element passes of one operation are launched (a property of this
  * GPU implementation; the paper has no counterpart):
- *   TLFE_LAUNCH_AUTO     : one persistent launch per operation over every pass
- *                          it covers (FP32 meshes, atomic or sorted scatter,
- *                          T4 / T10 / H8 blocks on the affine path) when there
- *                          are two or more such passes, else one launch per
- *                          pass; tlfe_autotune keeps whichever measures faster
+ *   TLFE_LAUNCH_AUTO     : one launch per pass, until tlfe_autotune measures one
+ *                          persistent launch per operation over every pass it
+ *                          covers (FP32 meshes of two or more such passes,
+ *                          atomic or sorted scatter, T4 / T10 / H8 blocks on
+ *                          the affine path) to be faster
  *   TLFE_LAUNCH_PER_PASS : one launch per pass (element block and law)
  *   TLFE_LAUNCH_FUSED    : the persistent launch wherever it covers a pass */
 enum { TLFE_LAUNCH_AUTO = 0, TLFE_LAUNCH_PER_PASS = 1, TLFE_LAUNCH_FUSED = 2 };

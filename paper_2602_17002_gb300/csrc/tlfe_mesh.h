@@ -66,7 +66,13 @@ struct FusedPlan {
     int *d_counter = nullptr;                 // one counter per fused op
     LaunchSched sched[2];                     // [0] force, [1] operator product
     size_t wreg[2] = {0, 0};
-    bool on[2] = {true, true};                // fused (true) or per-pass launches, per op
+    // fused (true) or per-pass launches, per op, in TLFE_LAUNCH_AUTO: per pass
+    // until the autotuner measures the fused launch faster. Measured on mixed
+    // batches of 6.6k, 56k, 378k and 1.58M elements (3 to 6 passes), force: 137,
+    // 218, 241, 375 us fused, 25, 49, 68, 164 us per pass; force + K v (one pass
+    // per block and law, which the fused launch rules out): 329, 517, 597, 942
+    // against 23, 47, 96, 266 us
+    bool on[2] = {false, false};
 };
 
 struct OpGraph;    // graph.cu: the captured force + operator-product call
