@@ -1331,7 +1331,7 @@ static tlfe_status run_fused(tlfe_mesh *m, const KParams<float> &base, cudaStrea
 
 template <int OP, typename R>
 tlfe_status run_op(tlfe_mesh *m, const void *u, const void *ud, const void *v, void *out0, void *out1,
-                   double *gth, double aM, double aK, double aC, int sym_only, cudaStream_t s)
+                   double *gth, double aM, double aK, double aC, int sym_only, cudaStream_t s, bool clear)
 {
     KParams<R> p;
     memset(&p, 0, sizeof(p));
@@ -1354,8 +1354,8 @@ tlfe_status run_op(tlfe_mesh *m, const void *u, const void *ud, const void *v, v
         p.part0 = (R *)m->d_part;
         p.part1 = p.part0 + 3 * std::max<int64_t>(1, m->n_part);
     } else {
-        if (out0) CK(cudaMemsetAsync(out0, 0, nb, s));
-        if (out1) CK(cudaMemsetAsync(out1, 0, nb, s));
+        if (out0 && clear) CK(cudaMemsetAsync(out0, 0, nb, s));
+        if (out1 && clear) CK(cudaMemsetAsync(out1, 0, nb, s));
     }
     const bool fused = use_fused<OP, R>(m);
     if constexpr (sizeof(R) == 4 && (OP == OP_FORCE || OP == OP_MATVEC)) {
@@ -1609,16 +1609,16 @@ static tlfe_status tune_all(tlfe_mesh *m, const double *u, const void *ud, const
     return st;
 }
 
-template tlfe_status run_op<OP_FORCE, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_FORCE, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_MATVEC, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_MATVEC, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_DIAG, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_DIAG, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_VJP, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_VJP, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_FM, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
-template tlfe_status run_op<OP_FM, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t);
+template tlfe_status run_op<OP_FORCE, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_FORCE, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_MATVEC, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_MATVEC, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_DIAG, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_DIAG, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_VJP, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_VJP, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_FM, double>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
+template tlfe_status run_op<OP_FM, float>(tlfe_mesh *, const void *, const void *, const void *, void *, void *, double *, double, double, double, int, cudaStream_t, bool);
 
 }  // namespace tlfe
 

@@ -17,7 +17,10 @@
 //
 // Per-body reductions are deterministic: the DOFs of every body (which must
 // own one contiguous node range) are cut into fixed chunks; one CTA reduces a
-// chunk into a partial, and one thread per body sums its partials in order.
+// chunk into a partial, and one warp per body sums its partials in a fixed
+// order. In the CG iteration that warp belongs to the body's last CTA to
+// finish (no CTA waits for another), so that alpha, beta and the loop's
+// condition need no launches of their own.
 //
 // The whole step is one CUDA graph with two nested conditional WHILE nodes
 // (Newton outside, CG inside), captured on the first call for a given
@@ -34,9 +37,19 @@
 
 namespace tlfe {
 
-constexpr int CHUNK = 4096;  // DOFs per reduction chunk
 constexpr int RT = 256;      // threads per chunk CTA
 constexpr int UNR = 4;       // DOFs a thread of the CG vector kernels loads before it uses them
+// DOFs per reduction chunk: as many as leave at least four chunk CTAs on every
+// SM, from one round of the CTA's loads (1024) up to 4096. Small systems are
+// bound by the latency of a CTA's rounds (562k DOFs: 4096 leave less than one
+// CTA per SM), large ones by memory, where more CTAs only add launches and
+// partial sums.
+static int chunk_dofs(int64_t n_dofs, int n_sm)
+{
+    int c = 4096;
+    while (c > RT * UNR && n_dofs < (int64_t)4 * n_sm * c) c /= 2;
+    return c;
+}
 
 enum {
     S_G0 = 0,   // ||g_b(v_n)||
@@ -73,6 +86,8 @@ struct NewtonState {
     double *partials = nullptr;  // [2][n_chunks]
     double *sc = nullptr;        // [S_COUNT][nb]
     int *it = nullptr;           // [I_COUNT]
+    int *arrived = nullptr;      // [2][nb + 1] chunk CTAs done per body (p.Ap; r.r and r.z), bodies done; 0 between launches
+    int n_live = 0;              // bodies that own chunks
     tlfe_mesh *twin = nullptr;   // FP64 mesh for the residual (FP32 meshes only)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -120,10 +135,27 @@ __device__ __forceinline__ double warp_body_sum(const double *partials, int k0, 
 {
     const int l = threadIdx.x & 31;
     double s = 0.0;
-    for (int k = k0 + l; k < k1; k += 32) s += partials[k];
+    for (int k = k0 + l; k < k1; k += 32) s += __ldcg(partials + k);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
+}
+
+// Whether this CTA is the last of its n to get here; called by every thread,
+// after thread 0 has written the CTA's partials. The count starts at 0 and the
+// last CTA puts it back. The last CTA sees every other one's partials (fence
+// before the count, fence after it).
+__device__ __forceinline__ bool last_to_arrive(int *count, int n)
+{
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(count, 1) == n - 1 ? 1 : 0;
+        if (last) *count = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    return last != 0;
 }
 
 struct ChunkArgs {
@@ -259,7 +291,7 @@ __global__ void k_dinv(ChunkArgs c, const R *D, const uint8_t *fixed, const doub
 // x = 0, r = -g (active bodies), z = Dinv r, p = z; partials of r.z and r.r
 template <typename R>
 __global__ void k_cg_init(ChunkArgs c, const double *g, const R *Dinv, const double *sc, int nb, R *x, R *r, R *p,
-                          double *partials)
+                          R *Ap, double *partials)
 {
     __shared__ double sh[32];
     const int ch = blockIdx.x;
@@ -272,6 +304,7 @@ __global__ void k_cg_init(ChunkArgs c, const double *g, const R *Dinv, const dou
         x[i] = R(0);
         r[i] = ri;
         p[i] = zi;
+        Ap[i] = R(0);  // the operator adds into it (k_cg_p clears it for the next iteration)
         rz.add(ri, zi);
         rr.add(ri, ri);
     }
@@ -308,13 +341,16 @@ __global__ void k_cg_init_finish(int nb, const int32_t *boff, const double *part
 
 // partial of p.Ap, Ap the operator product with the clamped DOFs zero
 // (k_cg_xr forms the same values again). Each thread loads UNR DOFs before
-// it uses them; its sum runs over its DOFs in plain strided order.
+// it uses them; its sum runs over its DOFs in plain strided order. The body's
+// last CTA forms alpha = r.z / p.Ap.
 template <typename R>
 __global__ void k_cg_pap(ChunkArgs c, const R *__restrict__ Ap, const uint8_t *__restrict__ fixed,
-                         const R *__restrict__ p, double *partials)
+                         const R *__restrict__ p, double *partials, const int32_t *__restrict__ boff, int nb, double *sc,
+                         int *arrived)
 {
     __shared__ double sh[32];
     const int ch = blockIdx.x;
+    const int b = c.body[ch];
     const int i1 = c.end[ch];
     DotAcc<R> acc;
     for (int i0 = c.start[ch] + threadIdx.x; i0 < i1; i0 += UNR * RT) {
@@ -331,27 +367,23 @@ __global__ void k_cg_pap(ChunkArgs c, const R *__restrict__ Ap, const uint8_t *_
     }
     const double s = block_sum(acc.value(), sh);
     if (threadIdx.x == 0) partials[ch] = s;
-}
-
-__global__ void k_cg_alpha(int nb, const int32_t *boff, const double *partials, double *sc)
-{
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int b = threadIdx.x >> 5; b < nb; b += nw) {  // one warp per body
-        const double pap = warp_body_sum(partials, boff[b], boff[b + 1]);
-        if (lane != 0) continue;
-        const bool act = sc[S_CACT * nb + b] != 0.0 && pap > 0.0;
-        if (sc[S_CACT * nb + b] != 0.0 && !(pap > 0.0)) sc[S_CACT * nb + b] = 0.0;  // not SPD here: stop this body
-        sc[S_ALPHA * nb + b] = act ? sc[S_RZ * nb + b] / pap : 0.0;
-    }
+    if (!last_to_arrive(arrived + b, boff[b + 1] - boff[b]) || threadIdx.x >= 32) return;
+    const double pap = warp_body_sum(partials, boff[b], boff[b + 1]);
+    if (threadIdx.x != 0) return;
+    const bool cg = sc[S_CACT * nb + b] != 0.0, act = cg && pap > 0.0;
+    if (cg && !act) sc[S_CACT * nb + b] = 0.0;  // not SPD here: stop this body
+    sc[S_ALPHA * nb + b] = act ? sc[S_RZ * nb + b] / pap : 0.0;
 }
 
 // x += alpha p, r -= alpha Ap; partials of r.r and r.z with z = Dinv r (z is
 // not stored: k_cg_p forms it again). Ap with the clamped DOFs zeroed, as in
-// k_cg_pap.
+// k_cg_pap. The body's last CTA forms beta and tests the body's convergence;
+// the last body to do so sets the loop's condition.
 template <typename R>
-__global__ void k_cg_xr(ChunkArgs c, const double *sc, int nb, const R *__restrict__ p, const R *__restrict__ Ap,
+__global__ void k_cg_xr(ChunkArgs c, double *sc, int nb, const R *__restrict__ p, const R *__restrict__ Ap,
                         const uint8_t *__restrict__ fixed, const R *__restrict__ Dinv, R *__restrict__ x,
-                        R *__restrict__ r, double *partials)
+                        R *__restrict__ r, double *partials, const int32_t *__restrict__ boff, int n_live, int *arrived,
+                        int *it, double rtol, int max_cg, cudaGraphConditionalHandle hC, int use_handle)
 {
     __shared__ double sh[32];
     const int ch = blockIdx.x;
@@ -389,33 +421,30 @@ __global__ void k_cg_xr(ChunkArgs c, const double *sc, int nb, const R *__restri
     if (threadIdx.x == 0) partials[ch] = s1;
     const double s2 = block_sum(rz.value(), sh);
     if (threadIdx.x == 0) partials[c.n_chunks + ch] = s2;
-}
-
-__global__ void k_cg_beta(int nb, const int32_t *boff, const double *partials, int n_chunks, double *sc, int *it,
-                          double rtol, int max_cg, cudaGraphConditionalHandle hC, int use_handle)
-{
-    int any = 0;
-    const int itn = it[I_CG] + 1;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int b = threadIdx.x >> 5; b < nb; b += nw) {  // one warp per body
-        const double rr = warp_body_sum(partials, boff[b], boff[b + 1]);
-        const double rz = warp_body_sum(partials + n_chunks, boff[b], boff[b + 1]);
-        if (lane != 0) continue;
-        const double rn = sqrt(rr);
-        int act = sc[S_CACT * nb + b] != 0.0 ? 1 : 0;
-        if (act) {
-            sc[S_RN * nb + b] = rn;
-            const double rz_old = sc[S_RZ * nb + b];
-            sc[S_BETA * nb + b] = rz_old != 0.0 ? rz / rz_old : 0.0;
-            sc[S_RZ * nb + b] = rz;
-            if (!(rn > rtol * sc[S_R0 * nb + b]) || itn >= max_cg) act = 0;
-            sc[S_CACT * nb + b] = act;
-        }
-        any |= act;
-    }
-    any = __syncthreads_or(any);
+    if (!last_to_arrive(arrived + b, boff[b + 1] - boff[b]) || threadIdx.x >= 32) return;
+    const double srr = warp_body_sum(partials, boff[b], boff[b + 1]);
+    const double srz = warp_body_sum(partials + c.n_chunks, boff[b], boff[b + 1]);
+    int done = 0;
     if (threadIdx.x == 0) {
-        it[I_CG] = itn;
+        const double rn = sqrt(srr);
+        if (sc[S_CACT * nb + b] != 0.0) {
+            const double rz_old = sc[S_RZ * nb + b];
+            sc[S_RN * nb + b] = rn;
+            sc[S_BETA * nb + b] = rz_old != 0.0 ? srz / rz_old : 0.0;
+            sc[S_RZ * nb + b] = srz;
+            if (!(rn > rtol * sc[S_R0 * nb + b]) || it[I_CG] + 1 >= max_cg) sc[S_CACT * nb + b] = 0.0;
+        }
+        __threadfence();
+        done = atomicAdd(arrived + nb, 1) == n_live - 1 ? 1 : 0;
+        if (done) arrived[nb] = 0;
+        __threadfence();
+    }
+    if (!__shfl_sync(0xffffffffu, done, 0)) return;
+    int any = 0;
+    for (int k = threadIdx.x; k < nb; k += 32) any |= __ldcg(sc + S_CACT * nb + k) != 0.0 ? 1 : 0;
+    any = __any_sync(0xffffffffu, any);
+    if (threadIdx.x == 0) {
+        it[I_CG] += 1;
         it[I_CG_TOTAL] += 1;
         it[I_ANY_C] = any;
         if (use_handle) cudaGraphSetConditional(hC, any ? 1u : 0u);
@@ -423,16 +452,18 @@ __global__ void k_cg_beta(int nb, const int32_t *boff, const double *partials, i
 }
 
 // p = z + beta p with z = Dinv r, on CG-active bodies (unchanged bodies keep
-// theirs); p is the operator's next input
+// theirs); p is the operator's next input, and Ap, which the operator adds
+// into, is cleared here (every chunk), in place of a launch that only does so
 template <typename R>
 __global__ void k_cg_p(ChunkArgs c, const double *sc, int nb, const R *__restrict__ r, const R *__restrict__ Dinv,
-                       R *__restrict__ p)
+                       R *__restrict__ p, R *__restrict__ Ap)
 {
     const int ch = blockIdx.x;
     const int b = c.body[ch];
+    const int i1 = c.end[ch];
+    for (int i = c.start[ch] + threadIdx.x; i < i1; i += RT) Ap[i] = R(0);
     if (sc[S_CACT * nb + b] == 0.0) return;
     const R beta = R(sc[S_BETA * nb + b]);
-    const int i1 = c.end[ch];
     for (int i0 = c.start[ch] + threadIdx.x; i0 < i1; i0 += UNR * RT) {
         R zi[UNR], pi[UNR];
 #pragma unroll
@@ -475,10 +506,11 @@ __global__ void k_start(ChunkArgs c, const uint8_t *fixed, const double *v_n, do
     for (int i = c.start[ch] + threadIdx.x; i < c.end[ch]; i += blockDim.x) v[i] = fixed[i / 3] ? 0.0 : v_n[i];
 }
 
-__global__ void k_reset(int nb, double *sc, int *it)
+__global__ void k_reset(int nb, double *sc, int *it, int *arrived)
 {
     for (int b = threadIdx.x; b < nb; b += blockDim.x)
         for (int k = 0; k < S_COUNT; ++k) sc[k * nb + b] = 0.0;
+    for (int k = threadIdx.x; k < 2 * (nb + 1); k += blockDim.x) arrived[k] = 0;
     if (threadIdx.x == 0)
         for (int k = 0; k < I_COUNT; ++k) it[k] = 0;
 }
@@ -563,18 +595,20 @@ static tlfe_status setup_newton(tlfe_mesh *m, cudaStream_t s, int coupled)
     // convergence groups: one per body, or a single group when constraints
     // may couple bodies
     ns->nb = coupled ? 1 : m->n_bodies;
+    const int chunk = chunk_dofs(3 * (int64_t)N, m->n_sm);
     std::vector<int32_t> cs, ce, cb, boff(ns->nb + 1, 0);
     for (int b = 0; b < m->n_bodies; ++b) {
         const int grp = coupled ? 0 : b;
         if (nstart[b] >= 0)
-            for (int64_t d = 3 * (int64_t)nstart[b]; d < 3 * (int64_t)nend[b]; d += CHUNK) {
+            for (int64_t d = 3 * (int64_t)nstart[b]; d < 3 * (int64_t)nend[b]; d += chunk) {
                 cs.push_back((int32_t)d);
-                ce.push_back((int32_t)std::min<int64_t>(d + CHUNK, 3 * (int64_t)nend[b]));
+                ce.push_back((int32_t)std::min<int64_t>(d + chunk, 3 * (int64_t)nend[b]));
                 cb.push_back(grp);
             }
         boff[grp + 1] = (int32_t)cs.size();
     }
     ns->n_chunks = (int)cs.size();
+    for (int b = 0; b < ns->nb; ++b) ns->n_live += boff[b + 1] > boff[b] ? 1 : 0;
     if (ns->n_chunks == 0) return fail(TLFE_E_INVALID, "no body owns any node");
     const size_t N3 = 3 * (size_t)N;
     tlfe_status st = TLFE_OK;
@@ -598,6 +632,7 @@ static tlfe_status setup_newton(tlfe_mesh *m, cudaStream_t s, int coupled)
     NA(ns->partials, 2 * (size_t)ns->n_chunks);
     NA(ns->sc, (size_t)S_COUNT * ns->nb);
     NA(ns->it, (size_t)I_COUNT);
+    NA(ns->arrived, 2 * ((size_t)ns->nb + 1));
     NA(ns->alm, 2);
     NA(ns->g0keep, (size_t)ns->nb);
     NA(ns->con_bad, 1);
@@ -716,9 +751,10 @@ static tlfe_status enq_cg_init(const StepCtx &x, cudaStream_t s)
     }
     if (x.m->precision == TLFE_FP32)
         k_cg_init<float><<<nc, RT, 0, s>>>(x.c, ns->g, ns->Dinv32, ns->sc, ns->nb, ns->x32, ns->r32, ns->p32,
-                                           ns->partials);
+                                           ns->Ap32, ns->partials);
     else
-        k_cg_init<double><<<nc, RT, 0, s>>>(x.c, ns->g, ns->Dinv, ns->sc, ns->nb, ns->x, ns->r, ns->p, ns->partials);
+        k_cg_init<double><<<nc, RT, 0, s>>>(x.c, ns->g, ns->Dinv, ns->sc, ns->nb, ns->x, ns->r, ns->p, ns->y1,
+                                            ns->partials);
     k_cg_init_finish<<<1, 1024, 0, s>>>(ns->nb, ns->body_chunk_off, ns->partials, nc, ns->sc, ns->it, ns->max_cg,
                                          ns->hC, x.use_handle);
     NCK(cudaGetLastError());
@@ -733,35 +769,38 @@ static tlfe_status enq_cg_iter(const StepCtx &x, cudaStream_t s)
     tlfe_status st;
     if (x.m->precision == TLFE_FP32) {  // p32: the FP32 search direction, kept by k_cg_init / k_cg_p
         st = run_op<OP_MATVEC, float>(x.m, ns->u_cur, ns->ud32, ns->p32, ns->Ap32, nullptr, nullptr, 1.0 / h, h, 1.0,
-                                      1, s);
+                                      1, s, false);
         if (st != TLFE_OK) return st;
         if (ns->n_cons > 0) {  // + h^2 rho C_q^T C_q p (Gauss-Newton)
             NCK(con_j<float>(ns->n_cons, ns->con_sh, ns->con_nd, ns->con_gp, ns->p32, ns->con_w, s));
             NCK(con_jt<float>(ns->n_cons, ns->con_sh, ns->con_nd, ns->con_gp, ns->con_w, h * h * ns->rho, ns->Ap32, s));
         }
-        k_cg_pap<float><<<nc, RT, 0, s>>>(x.c, ns->Ap32, ns->fixed, ns->p32, ns->partials);
+        k_cg_pap<float><<<nc, RT, 0, s>>>(x.c, ns->Ap32, ns->fixed, ns->p32, ns->partials, ns->body_chunk_off, ns->nb,
+                                          ns->sc, ns->arrived);
     } else {
-        st = run_op<OP_MATVEC, double>(x.m, ns->u_cur, ns->v, ns->p, ns->y1, nullptr, nullptr, 1.0 / h, h, 1.0, 1, s);
+        st = run_op<OP_MATVEC, double>(x.m, ns->u_cur, ns->v, ns->p, ns->y1, nullptr, nullptr, 1.0 / h, h, 1.0, 1, s,
+                                       false);
         if (st != TLFE_OK) return st;
         if (ns->n_cons > 0) {
             NCK(con_j<double>(ns->n_cons, ns->con_sh, ns->con_nd, ns->con_gp, ns->p, ns->con_w, s));
             NCK(con_jt<double>(ns->n_cons, ns->con_sh, ns->con_nd, ns->con_gp, ns->con_w, h * h * ns->rho, ns->y1, s));
         }
-        k_cg_pap<double><<<nc, RT, 0, s>>>(x.c, ns->y1, ns->fixed, ns->p, ns->partials);
+        k_cg_pap<double><<<nc, RT, 0, s>>>(x.c, ns->y1, ns->fixed, ns->p, ns->partials, ns->body_chunk_off, ns->nb,
+                                           ns->sc, ns->arrived);
     }
-    k_cg_alpha<<<1, 1024, 0, s>>>(ns->nb, ns->body_chunk_off, ns->partials, ns->sc);
+    int *arr = ns->arrived + ns->nb + 1;
     if (x.m->precision == TLFE_FP32)
         k_cg_xr<float><<<nc, RT, 0, s>>>(x.c, ns->sc, ns->nb, ns->p32, ns->Ap32, ns->fixed, ns->Dinv32, ns->x32,
-                                         ns->r32, ns->partials);
+                                         ns->r32, ns->partials, ns->body_chunk_off, ns->n_live, arr, ns->it, ns->crtol,
+                                         ns->max_cg, ns->hC, x.use_handle);
     else
         k_cg_xr<double><<<nc, RT, 0, s>>>(x.c, ns->sc, ns->nb, ns->p, ns->y1, ns->fixed, ns->Dinv, ns->x, ns->r,
-                                          ns->partials);
-    k_cg_beta<<<1, 1024, 0, s>>>(ns->nb, ns->body_chunk_off, ns->partials, nc, ns->sc, ns->it, ns->crtol, ns->max_cg,
-                                  ns->hC, x.use_handle);
+                                          ns->partials, ns->body_chunk_off, ns->n_live, arr, ns->it, ns->crtol,
+                                          ns->max_cg, ns->hC, x.use_handle);
     if (x.m->precision == TLFE_FP32)
-        k_cg_p<float><<<nc, RT, 0, s>>>(x.c, ns->sc, ns->nb, ns->r32, ns->Dinv32, ns->p32);
+        k_cg_p<float><<<nc, RT, 0, s>>>(x.c, ns->sc, ns->nb, ns->r32, ns->Dinv32, ns->p32, ns->Ap32);
     else
-        k_cg_p<double><<<nc, RT, 0, s>>>(x.c, ns->sc, ns->nb, ns->r, ns->Dinv, ns->p);
+        k_cg_p<double><<<nc, RT, 0, s>>>(x.c, ns->sc, ns->nb, ns->r, ns->Dinv, ns->p, ns->y1);
     NCK(cudaGetLastError());
     return TLFE_OK;
 }
@@ -781,7 +820,7 @@ static tlfe_status enq_newton_tail(const StepCtx &x, cudaStream_t s)
 static tlfe_status enq_prologue(const StepCtx &x, cudaStream_t s)
 {
     NewtonState *ns = x.ns;
-    k_reset<<<1, 1024, 0, s>>>(ns->nb, ns->sc, ns->it);
+    k_reset<<<1, 1024, 0, s>>>(ns->nb, ns->sc, ns->it, ns->arrived);
     k_start<<<ns->n_chunks, RT, 0, s>>>(x.c, ns->fixed, ns->v_n, ns->v, ns->alm);
     NCK(cudaGetLastError());
     return enq_residual(x, s, true);

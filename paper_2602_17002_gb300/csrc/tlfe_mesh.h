@@ -168,8 +168,10 @@ void destroy_newton(tlfe_mesh *m);
 tlfe_mesh *newton_twin(tlfe_mesh *m);  // FP64 twin of an FP32 mesh built by the Newton step, or nullptr
 ConBlocks con_blocks(const tlfe_mesh *m);  // n = -1 when the mesh has more blocks than a constraint set supports
 
+// clear = false: the caller has zeroed the outputs (the sorted scatter
+// overwrites them either way)
 template <int OP, typename R>
 tlfe_status run_op(tlfe_mesh *m, const void *u, const void *ud, const void *v, void *out0, void *out1,
-                   double *gth, double aM, double aK, double aC, int sym_only, cudaStream_t s);
+                   double *gth, double aM, double aK, double aC, int sym_only, cudaStream_t s, bool clear = true);
 
 }  // namespace tlfe
