@@ -1626,7 +1626,11 @@ template <int OP, typename R> size_t region_for(int et, int umax, int meta_bytes
 template <int OP, typename R>
 size_t smem_for(int et, int nq, int umax, int meta_bytes, int wpb, bool aff, int mat, bool mass)
 {
-    if (wpe_path(et, aff)) return OP == OP_FM ? 0 : wpe_smem_bytes<R>(wpb);
+    if constexpr (OP == OP_FM) {
+        if (wpe_path(et, aff)) return 0;
+    } else {
+        if (wpe_path(et, aff)) return wpe_smem_bytes<R, OP>(wpb);
+    }
     if (pw_path(et, aff, OP, sizeof(R) == 4)) return pw_smem_for<OP>(nq, umax, meta_bytes);
     const size_t w = region_for<OP, R>(et, umax, meta_bytes, aff, mat, mass);
     return w ? cta_smem_bytes(w, wpb) : 0;
