@@ -369,23 +369,21 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 }
 
 // Resident CTAs (of 4 warps) per SM the register allocation aims at, by
-// measurement on the beam workload: the FP32 affine force kernel fits 16
-// warps per SM in 128 registers; the adjoint, with two element vectors live,
-// fits 12 warps in 168 registers (its local indices, J^{-1} and node 0's
-// pair re-read from shared memory at every point) without spill or with a
-// few bytes for the laws listed below, and runs 7 % faster there than at 8
-// warps and 214 registers; with the generic law or the undamped
-// neo-Hookean one it would spill 70-200 bytes and keeps 8 warps. FP64 kernels take all 255 registers,
-// and so do Q27 kernels (81-entry element vectors; their shared-memory
-// footprint limits the resident warps anyway).
+// measurement. Column paths (affine T10 and H8): 12 warps in 168 registers
+// with at most a few spilled values, the force 16 warps in 128; the generic
+// law keeps 8 warps and all its registers. Slab T10 adjoint and force +
+// operator product: 8 warps at 255 registers; at 12 warps they spill 150-210
+// bytes and the curved T10 step (194k elements) takes 158 us instead of 137.
+// T4, and H8 on the slab: 12 warps where the law's state fits 168 registers.
+// FP64 kernels take all 255 registers, and so do Q27 kernels (81-entry element
+// vectors; their shared-memory footprint limits the resident warps anyway).
 template <int ET, typename R, int OP, bool AFF, int MAT> constexpr int min_ctas()
 {
     if (sizeof(R) != 4 || ET == ET_Q27) return 1;
     if (t10_path<R>(ET, OP, AFF) || h8_path<R>(ET, OP, AFF)) return OP == OP_FORCE ? 4 : (MAT == MAT_ANY ? 2 : 3);
     if (OP == OP_VJP || OP == OP_FM) {
-        const bool fits = ET == ET_T4 || MAT == MAT_NH_KV || MAT == MAT_SVK || (MAT == MAT_SVK_KV && AFF) ||
-                          (ET == ET_H8 && MAT != MAT_ANY);
-        return fits ? 3 : 2;
+        if (ET == ET_T10) return 2;
+        return ET == ET_T4 || MAT != MAT_ANY ? 3 : 2;
     }
     return (OP == OP_FORCE && AFF) ? 4 : 3;
 }
