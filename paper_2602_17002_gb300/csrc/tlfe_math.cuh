@@ -10,7 +10,8 @@
 // Every law is evaluated through its second Piola-Kirchhoff stress S, P = F S:
 // S and its derivative are symmetric (6 entries), the elastic and the viscous
 // part share one product with F, and the derivative along dF needs two 3x3
-// products, dP = dF S + F dS, with dS linear in dE = sym(F^T dF). With
+// products, dP = dF S + F dS, with dS linear in dE = sym(F^T dF); F enters as
+// I + G term by term, so that its unit diagonal is never rounded. With
 // P = A cof(F) (first Piola-Kirchhoff form) the neo-Hookean + Kelvin-Voigt
 // stress and its derivative took about 515 multiply-adds a point instead of
 // about 350.
@@ -28,8 +29,8 @@
 // alpha2 = 2 mu01 J^{-10/3}, beta = k (J - 1) / J. M and Q are both sums of I
 // and N = B - cof(B): with s = 1 + t/3 and i = I2 + I3 - t (1 + t)/3,
 //   M = s N + i I, Q = (1 + t) I - N,
-//   S = (alpha s - beta) N + (alpha i + beta (1 + t)) I      (+ alpha2 M2),
-// and the same holds for the parts of dS that M and Q enter: neither is formed.
+//   S = (alpha s - beta) N + (alpha i + beta (1 + t)) I      (+ alpha2 M2):
+// neither is formed, and dS is the derivative of this form.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -167,6 +168,16 @@ template <typename V> __device__ __forceinline__ void sym_eng(const V A[9], cons
     e[5] = A[1] * B[2] + A[4] * B[5] + A[7] * B[8] + A[2] * B[1] + A[5] * B[4] + A[8] * B[7];
 }
 
+// eng(F, D) for F = I + G from G: no rounding of F's unit diagonal
+template <typename V> __device__ __forceinline__ void sym_eng_ig(const V G[9], const V D[9], V e[6])
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a) e[a] = D[4 * a] + G[a] * D[a] + G[3 + a] * D[3 + a] + G[6 + a] * D[6 + a];
+    e[3] = D[1] + D[3] + G[0] * D[1] + G[3] * D[4] + G[6] * D[7] + G[1] * D[0] + G[4] * D[3] + G[7] * D[6];
+    e[4] = D[2] + D[6] + G[0] * D[2] + G[3] * D[5] + G[6] * D[8] + G[2] * D[0] + G[5] * D[3] + G[8] * D[6];
+    e[5] = D[5] + D[7] + G[1] * D[2] + G[4] * D[5] + G[7] * D[8] + G[2] * D[1] + G[5] * D[4] + G[8] * D[7];
+}
+
 // S : e for a symmetric S and an engineering e (the doubled off-diagonals are in e)
 template <typename V> __device__ __forceinline__ V dot6(const V S[6], const V e[6])
 {
@@ -197,54 +208,70 @@ template <typename V> __device__ __forceinline__ void dcof6(const V C[6], const 
     d[5] = C[3] * e[4] + C[4] * e[3] - C[0] * e[5] - C[5] * t0;
 }
 
-// P = A S with S symmetric (6 entries)
+// Products with a symmetric S (6 entries): P = A S, P += A S, and P = F S for
+// F = I + G, as S + G S (no rounding of F's unit diagonal)
+template <typename V> __device__ __forceinline__ void full6(const V S[6], V M[9])
+{
+    M[0] = S[0], M[4] = S[1], M[8] = S[2];
+    M[1] = M[3] = S[3];
+    M[2] = M[6] = S[4];
+    M[5] = M[7] = S[5];
+}
 template <typename V> __device__ __forceinline__ void mm6(const V A[9], const V S[6], V P[9])
 {
+    V M[9];
+    full6(S, M);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        P[a * 3 + 0] = A[a * 3] * S[0] + A[a * 3 + 1] * S[3] + A[a * 3 + 2] * S[4];
-        P[a * 3 + 1] = A[a * 3] * S[3] + A[a * 3 + 1] * S[1] + A[a * 3 + 2] * S[5];
-        P[a * 3 + 2] = A[a * 3] * S[4] + A[a * 3 + 1] * S[5] + A[a * 3 + 2] * S[2];
-    }
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) P[a * 3 + b] = A[a * 3] * M[b] + A[a * 3 + 1] * M[3 + b] + A[a * 3 + 2] * M[6 + b];
 }
 template <typename V> __device__ __forceinline__ void mm6_acc(const V A[9], const V S[6], V P[9])
 {
+    V M[9];
+    full6(S, M);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        P[a * 3 + 0] += A[a * 3] * S[0] + A[a * 3 + 1] * S[3] + A[a * 3 + 2] * S[4];
-        P[a * 3 + 1] += A[a * 3] * S[3] + A[a * 3 + 1] * S[1] + A[a * 3 + 2] * S[5];
-        P[a * 3 + 2] += A[a * 3] * S[4] + A[a * 3 + 1] * S[5] + A[a * 3 + 2] * S[2];
-    }
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            P[a * 3 + b] = P[a * 3 + b] + A[a * 3] * M[b] + A[a * 3 + 1] * M[3 + b] + A[a * 3 + 2] * M[6 + b];
 }
 // FP32: rows 0 and 1 paired in packed FP32x2 operations (one issue slot for
 // two multiply-adds; broadcast and swapped operands are free)
 __device__ __forceinline__ void mm6(const float A[9], const float S[6], float P[9])
 {
     const float2 a0 = make_float2(A[0], A[3]), a1 = make_float2(A[1], A[4]), a2 = make_float2(A[2], A[5]);
-    const float s[9] = {S[0], S[3], S[4], S[3], S[1], S[5], S[4], S[5], S[2]};
+    float M[9];
+    full6(S, M);
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        float2 q = __fmul2_rn(a0, make_float2(s[b], s[b]));
-        q = __ffma2_rn(a1, make_float2(s[3 + b], s[3 + b]), q);
-        q = __ffma2_rn(a2, make_float2(s[6 + b], s[6 + b]), q);
+        float2 q = __fmul2_rn(a0, make_float2(M[b], M[b]));
+        q = __ffma2_rn(a1, make_float2(M[3 + b], M[3 + b]), q);
+        q = __ffma2_rn(a2, make_float2(M[6 + b], M[6 + b]), q);
         P[b] = q.x;
         P[3 + b] = q.y;
-        P[6 + b] = fmaf(A[8], s[6 + b], fmaf(A[7], s[3 + b], A[6] * s[b]));
+        P[6 + b] = fmaf(A[8], M[6 + b], fmaf(A[7], M[3 + b], A[6] * M[b]));
     }
 }
 __device__ __forceinline__ void mm6_acc(const float A[9], const float S[6], float P[9])
 {
     const float2 a0 = make_float2(A[0], A[3]), a1 = make_float2(A[1], A[4]), a2 = make_float2(A[2], A[5]);
-    const float s[9] = {S[0], S[3], S[4], S[3], S[1], S[5], S[4], S[5], S[2]};
+    float M[9];
+    full6(S, M);
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        float2 q = __ffma2_rn(a0, make_float2(s[b], s[b]), make_float2(P[b], P[3 + b]));
-        q = __ffma2_rn(a1, make_float2(s[3 + b], s[3 + b]), q);
-        q = __ffma2_rn(a2, make_float2(s[6 + b], s[6 + b]), q);
+        float2 q = __ffma2_rn(a0, make_float2(M[b], M[b]), make_float2(P[b], P[3 + b]));
+        q = __ffma2_rn(a1, make_float2(M[3 + b], M[3 + b]), q);
+        q = __ffma2_rn(a2, make_float2(M[6 + b], M[6 + b]), q);
         P[b] = q.x;
         P[3 + b] = q.y;
-        P[6 + b] = fmaf(A[8], s[6 + b], fmaf(A[7], s[3 + b], fmaf(A[6], s[b], P[6 + b])));
+        P[6 + b] = fmaf(A[8], M[6 + b], fmaf(A[7], M[3 + b], fmaf(A[6], M[b], P[6 + b])));
     }
+}
+template <typename V> __device__ __forceinline__ void mm6_ig(const V G[9], const V S[6], V P[9])
+{
+    full6(S, P);
+    mm6_acc(G, S, P);
 }
 
 // ---------------------------------------------------------------------------
@@ -254,8 +281,7 @@ __device__ __forceinline__ void mm6_acc(const float A[9], const float S[6], floa
 // Per-point quantities kept between the stress and its derivatives (V: one
 // point, or two of one element in F2).
 template <typename V> struct QP {
-    V F[9];    // I + G
-    V G[9];    // sum u_i h_i^T
+    V G[9];    // sum u_i h_i^T; F = I + G
     V Fd[9];   // sum udot_i h_i^T (valid when visc)
     V S[6];    // elastic second Piola-Kirchhoff stress
     V Sv[6];   // viscous second Piola-Kirchhoff stress (valid when visc)
@@ -289,13 +315,11 @@ __device__ __forceinline__ void mr_factors(V t, V I2, V I3, V &x0, V &x1, V &x2)
 template <typename R, typename V> __device__ __forceinline__ void stress_state(const Mat<R> &m, QP<V> &q, bool visc)
 {
     const V *G = q.G;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) q.F[k] = k % 4 == 0 ? G[k] + V(R(1)) : G[k];
     set_true(q.ok);
     if (visc) {
         // Edot = sym(Fd^T F); S^v = 2 mu_v Edot + lam_v tr(Edot) I  (Sec. 3.2.3)
         V e[6];
-        sym_eng<V>(q.Fd, q.F, e);
+        sym_eng_ig<V>(G, q.Fd, e);
         const V i = m.lam_v * (e[0] + e[1] + e[2]);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -326,13 +350,19 @@ template <typename R, typename V> __device__ __forceinline__ void stress_state(c
     const V dG = G[0] * c0 + G[1] * c1 + G[2] * c2;
     const V I2G = c0 + (G[0] * G[4] - G[1] * G[3]) + (G[0] * G[8] - G[2] * G[6]);
     const V Jm1 = (G[0] + G[4] + G[8]) + I2G + dG;
-    const V J = Jm1 + V(R(1));
-    q.ok = positive(J);
-    const V r = rcbrt_(where(q.ok, J, V(R(1)))), r2 = r * r;
+    q.ok = positive(Jm1 + V(R(1)));
+    const V jm = where(q.ok, Jm1, V(R(0))), J = jm + V(R(1));
+    // J^{-1/3} and 1/J to the last bit of 1 + (J - 1): alpha holds the eighth
+    // power of J^{-1/3}, whose rounding (and that of J) would otherwise be most
+    // of the FP32 error of the operator product. err = 1 - r^3 (J + jl).
+    const V r0 = rcbrt_(J), rJ0 = V(r0 * r0) * r0;
+    const V jl = jm - (J - V(R(1)));
+    const V err = V(V(R(1)) - rJ0 * J) - rJ0 * jl;
+    const V r = r0 + V(third * r0) * err, r2 = r * r;
     q.r1 = r;
-    q.rJ = r2 * r;
+    q.rJ = rJ0 + rJ0 * err;
     q.rD = q.rJ * q.rJ;
-    q.Jm1r = Jm1 * q.rJ;
+    q.Jm1r = jm * q.rJ;
     q.al = (m.mu - R(2) * m.mu01) * V(q.rD * r2);
     const V be = (m.lam + R(2) * third * m.mu) * q.Jm1r;
     V cB[6];
@@ -384,7 +414,7 @@ template <typename V> __device__ __forceinline__ void first_piola(const QP<V> &q
     V St[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) St[k] = visc ? q.S[k] + q.Sv[k] : q.S[k];
-    mm6(q.F, St, P);
+    mm6_ig(q.G, St, P);
     if (!all_of(q.ok) && !visc)  // an F that is not a number leaves no trace
 #pragma unroll
         for (int k = 0; k < 9; ++k) P[k] = where(q.ok, P[k], V(R(0)));
@@ -412,29 +442,30 @@ __device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<V> &q, cons
         }
         return;
     }
-    // S_iso = alpha M = mu J^{-2/3} (I - I1/3 C^{-1}), C^{-1} = Q / J^2, j = dJ / J = C^{-1} : dE:
-    //   dS_iso = -(2/3) j S_iso - mu J^{-2/3}/3 (2 tr dE C^{-1} + I1 dC^{-1})
-    //   d(k (J - 1) J C^{-1}) = k (2J - 1) J j C^{-1} + k (J - 1) J dC^{-1}
-    //   dC^{-1} = (dQ - 2 j Q) / J^2
+    // derivative of S = c1 N + c0 I, c1 = alpha s - beta, c0 = alpha i + beta (1 + t), along dB = 2 dE
+    // (j = dJ / J = Q : dE / J^2, dt = 2 tr dE; dalpha = -8/3 alpha j, dbeta = k j / J):
+    //   dN = dB - dcof(B), ds = dt / 3, di = dt (t - 1) / 3 - 2 N : dE
+    // No term is larger than the derivative itself (formed from M, Q and dcof(C), whose identity parts
+    // cancel, the FP32 error is 1.4 times as large).
     const R third = R(1.0 / 3.0);
     const R kb = m.lam + R(2) * third * m.mu;
-    const V QE = q.t1 * trE - dot6<V>(q.N, e);
-    const V j = QE * q.rD;
-    const V a23 = (c * R(2) * third) * q.al;
-    const V xM = a23 * -j;
-    const V cj = c * j;
-    // alpha s is alpha I1 / 3; beta = alpha s - c1
-    const V xQ = cj * (q.al * q.s + q.c1 + V(kb)) - a23 * trE;
-    const V xd = -c * q.c1;
-    const V xd2 = xd + xd;
-    const V y1 = xM * q.s - xQ, y0 = xM * q.i + xQ * q.t1;
-    V C[6], dQ[6];
+    const V NE = dot6<V>(q.N, e);
+    const V dt = trE + trE;
+    const V j = (q.t1 * trE - NE) * q.rD;
+    const V da = V((R(-8) * third) * q.al) * j;   // dalpha
+    const V db = V(kb * j) * q.rJ;                // dbeta
+    const V adt = V(third * q.al) * dt;           // alpha dt / 3
+    const V be = q.al * q.s - q.c1;
+    const V dc1 = c * V(da * q.s + adt - db);
+    const V dc0 = c * V(da * q.i + adt * (q.t1 - V(R(2))) - V(q.al * (NE + NE)) + db * q.t1 + be * dt);
+    const V cc = c * q.c1, cc2 = cc + cc;
+    V d[6];
+    dcof6<V>(q.B, e, d);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) C[k] = k < 3 ? q.B[k] + V(R(1)) : q.B[k];
-    dcof6<V>(C, e, dQ);
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-        dS[k] = k < 3 ? V(y1 * q.N[k] + V(xd2 * dQ[k] + y0)) : V(y1 * q.N[k] + xd * dQ[k]);
+    for (int k = 0; k < 6; ++k) {
+        const V u = e[k] - d[k];
+        dS[k] = k < 3 ? V(cc2 * u + V(dc1 * q.N[k] + dc0)) : V(cc * u + dc1 * q.N[k]);
+    }
     if (m.model == MODEL_MR) {
         // S2 = a2 M2, a2 = 2 mu01 J^{-10/3}: dS2 = -(10/3) j S2 + a2 dM2
         const V t = q.B[0] + q.B[1] + q.B[2];
@@ -448,7 +479,6 @@ __device__ __forceinline__ void dS_elastic(const Mat<R> &m, const QP<V> &q, cons
         // invariants of B along dB = 2 dE
         V dcB[6];
         dcof6<V>(q.B, e, dcB);  // diagonal halved
-        const V dt = R(2) * trE;
         const V dI2 = R(2) * (dcB[0] + dcB[1] + dcB[2]);
         const V dI3 = R(2) * dot6<V>(cB, e);
         const V dx1 = third * (dt - dI2) - dI3;
@@ -476,10 +506,11 @@ template <typename R, typename V>
 __device__ __forceinline__ void dstress(const Mat<R> &m, const QP<V> &q, bool visc, const V dF[9],
                                         R cK, R cC, bool sym_only, V dP[9])
 {
-    V e[6], T[6];
-    sym_eng<V>(q.F, dF, e);
+    V e[6], T[6], Sk[6];
+    sym_eng_ig<V>(q.G, dF, e);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) T[k] = Sk[k] = V(R(0));
     if (cK != R(0)) {
-        V Sk[6];
         dS_elastic<R, V>(m, q, e, cK, T);
         const bool vk = visc && !sym_only;
         if (vk) {  // position-side viscous derivative: dEdot = sym(Fd^T dF)
@@ -495,12 +526,6 @@ __device__ __forceinline__ void dstress(const Mat<R> &m, const QP<V> &q, bool vi
         }
 #pragma unroll
         for (int k = 0; k < 6; ++k) Sk[k] = cK * (vk ? q.S[k] + q.Sv[k] : q.S[k]);
-        mm6(dF, Sk, dP);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) T[k] = V(R(0));
-#pragma unroll
-        for (int k = 0; k < 9; ++k) dP[k] = V(R(0));
     }
     if (cC != R(0)) {  // velocity direction: dEdot = sym(F^T dFd)
         const R a = cC * m.mu_v;
@@ -511,7 +536,8 @@ __device__ __forceinline__ void dstress(const Mat<R> &m, const QP<V> &q, bool vi
             T[3 + k] += a * e[3 + k];
         }
     }
-    mm6_acc(q.F, T, dP);
+    mm6_ig(q.G, T, dP);
+    if (cK != R(0)) mm6_acc(dF, Sk, dP);
     if (!all_of(q.ok) && !(visc && !sym_only) && !(cC != R(0) && (m.mu_v != R(0) || m.lam_v != R(0))))
 #pragma unroll
         for (int k = 0; k < 9; ++k) dP[k] = where(q.ok, dP[k], V(R(0)));
@@ -526,12 +552,12 @@ __device__ __forceinline__ void astress(const Mat<R> &m, const QP<V> &q, bool vi
                                         V gF[9], V gFd[9], V &gmu, V &glam)
 {
     V e[6], T[6], St[6];
-    sym_eng<V>(q.F, Gh, e);
+    sym_eng_ig<V>(q.G, Gh, e);
     dS_elastic<R, V>(m, q, e, R(1), T);
 #pragma unroll
     for (int k = 0; k < 6; ++k) St[k] = visc ? q.S[k] + q.Sv[k] : q.S[k];
-    mm6(Gh, St, gF);
-    mm6_acc(q.F, T, gF);
+    mm6_ig(q.G, T, gF);
+    mm6_acc(Gh, St, gF);
     const V trE = e[0] + e[1] + e[2];
     if (visc) {
         // L = (F S^v) : Gh, Ebar = 2 mu_v sym(F^T Gh) + lam_v tr I:
@@ -544,7 +570,7 @@ __device__ __forceinline__ void astress(const Mat<R> &m, const QP<V> &q, bool vi
             Eb[3 + k] = m.mu_v * e[3 + k];
         }
         mm6_acc(q.Fd, Eb, gF);
-        mm6(q.F, Eb, gFd);
+        mm6_ig(q.G, Eb, gFd);
     } else {
 #pragma unroll
         for (int k = 0; k < 9; ++k) gFd[k] = V(R(0));
