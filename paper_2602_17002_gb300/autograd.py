@@ -15,24 +15,25 @@ class InternalForce(torch.autograd.Function):
     def forward(ctx, mesh: Mesh, u, udot, theta):
         if theta is not None:
             mesh.set_elem_mu_lambda(theta.detach().contiguous())
-        f = mesh.internal_force(u.detach().double().contiguous(),
-                                None if udot is None else udot.detach().to(mesh.torch_dtype).contiguous())
+        # the state in the library's types; kept for the backward pass, with the
+        # inputs themselves, whose change in place between the two is an error
+        ul = u.detach().double().contiguous()
+        udl = None if udot is None else udot.detach().to(mesh.torch_dtype).contiguous()
+        f = mesh.internal_force(ul, udl)
         ctx.mesh = mesh
         ctx.has_udot = udot is not None
         ctx.has_theta = theta is not None
-        ctx.save_for_backward(u, udot if udot is not None else u, theta if theta is not None else u)
+        ctx.save_for_backward(u, udot if udot is not None else u, theta if theta is not None else u, ul, udl)
         return f
 
     @staticmethod
     def backward(ctx, gf):
-        u, udot, theta = ctx.saved_tensors
+        u, udot, theta, ul, udl = ctx.saved_tensors
         mesh = ctx.mesh
         if ctx.has_theta:
             mesh.set_elem_mu_lambda(theta.detach().contiguous())
         need_u, need_ud, need_th = ctx.needs_input_grad[1], ctx.needs_input_grad[2], ctx.needs_input_grad[3]
-        gu, gud, gth = mesh.vjp(u.detach().double().contiguous(),
-                                udot.detach().to(mesh.torch_dtype).contiguous() if ctx.has_udot else None,
-                                gf.detach().to(mesh.torch_dtype).contiguous(), want_u=True,
+        gu, gud, gth = mesh.vjp(ul, udl, gf.detach().to(mesh.torch_dtype).contiguous(), want_u=True,
                                 want_udot=need_ud, want_theta=need_th)
         if gu is not None:
             gu = gu.to(u.dtype)

@@ -185,21 +185,23 @@ def _check(code: int):
         raise TLFEError(code, load().tlfe_last_error().decode())
 
 
+# Streams and device pointers go to the library as plain integers (None: NULL);
+# ctypes converts them by the declared argument types. On small meshes the
+# binding is a large part of a call, so the current stream comes as its raw
+# handle, without a Stream object.
 def _stream(stream):
     if stream is None:
         import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
-        return C.c_void_p(stream)
-    return C.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return C.c_void_p(t)
-    return C.c_void_p(t.data_ptr())
+    if t is None or isinstance(t, int):
+        return t
+    return t.data_ptr()
 
 
 class Mesh:
@@ -360,8 +362,8 @@ class Mesh:
         if t is None:
             return None
         dt = dtype or self.torch_dtype
-        if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dt and t.is_contiguous()
-                and tuple(t.shape) == (self.n_nodes, 3)):
+        if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dt and t.shape == (self.n_nodes, 3)
+                and t.is_contiguous()):
             raise TLFEError(1, f"{name} must be a contiguous CUDA {dt} tensor of shape ({self.n_nodes}, 3)")
         return t
 
