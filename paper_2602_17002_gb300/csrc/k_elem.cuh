@@ -28,7 +28,11 @@
 //     16-byte load, hit distinct bank groups;
 //   - each lane evaluates F = I + sum_i u_i h_i^T per quadrature point and the
 //     stress, its directional derivative, its adjoint or the diagonal moduli,
-//     accumulating its element vector sum_q w_q J_p (.) h_iq in registers;
+//     accumulating its element vector sum_q w_q J_p (.) h_iq in registers. FP32
+//     affine T10 and H8 blocks (column_path) instead form the gradients from
+//     what their points share, keep them in the lane's own shared column and
+//     evaluate two points at a time (k_t10.cuh, k_h8.cuh); they read the
+//     per-lane tables of a tile straight from global memory;
 //   - element vectors go to shared slots in node-sorted positions (a list
 //     built at mesh creation); one lane per unique node sums that node's slots
 //     and adds the sum to the global array with one atomic per component (a
@@ -374,17 +378,22 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 // law keeps 8 warps and all its registers. Slab T10 adjoint and force +
 // operator product: 8 warps at 255 registers; at 12 warps they spill 150-210
 // bytes and the curved T10 step (194k elements) takes 158 us instead of 137.
+// The damped neo-Hookean law alone also gains by that in the slab T10 operator
+// product (65.0 -> 61.8 us) and in the H8 adjoint and one pass (step of 140k
+// bricks 111.0 -> 106.8 us; 86.7 -> 92.4 without damping).
 // T4, and H8 on the slab: 12 warps where the law's state fits 168 registers.
 // FP64 kernels take all 255 registers, and so do Q27 kernels (81-entry element
 // vectors; their shared-memory footprint limits the resident warps anyway).
 template <int ET, typename R, int OP, bool AFF, int MAT> constexpr int min_ctas()
 {
     if (sizeof(R) != 4 || ET == ET_Q27) return 1;
+    if (h8_path<R>(ET, OP, AFF) && (OP == OP_FM || OP == OP_VJP) && MAT == MAT_NH_KV) return 2;
     if (t10_path<R>(ET, OP, AFF) || h8_path<R>(ET, OP, AFF)) return OP == OP_FORCE ? 4 : (MAT == MAT_ANY ? 2 : 3);
     if (OP == OP_VJP || OP == OP_FM) {
         if (ET == ET_T10) return 2;
         return ET == ET_T4 || MAT != MAT_ANY ? 3 : 2;
     }
+    if (OP == OP_MATVEC && !AFF && ET == ET_T10 && MAT == MAT_NH_KV) return 2;
     return (OP == OP_FORCE && AFF) ? 4 : 3;
 }
 

@@ -126,8 +126,6 @@ __device__ __forceinline__ void set_true(Mask2 &m) { m.x = m.y = true; }
 // 3x3 helpers on row-major register arrays
 // ---------------------------------------------------------------------------
 
-template <typename R> __device__ __forceinline__ R tr3(const R A[9]) { return A[0] + A[4] + A[8]; }
-
 // R = A B
 template <typename R> __device__ __forceinline__ void mm3(const R A[9], const R B[9], R C[9])
 {
