@@ -378,9 +378,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 // law keeps 8 warps and all its registers. Slab T10 adjoint and force +
 // operator product: 8 warps at 255 registers; at 12 warps they spill 150-210
 // bytes and the curved T10 step (194k elements) takes 158 us instead of 137.
-// The damped neo-Hookean law alone also gains by that in the slab T10 operator
-// product (65.0 -> 61.8 us) and in the H8 adjoint and one pass (step of 140k
-// bricks 111.0 -> 106.8 us; 86.7 -> 92.4 without damping).
+// So too with damped Saint Venant-Kirchhoff (323k: 208 -> 195 us) and the
+// undamped neo-Hookean law (323k: 201 -> 195); undamped Saint Venant-Kirchhoff
+// spills little and keeps 12 warps (99k: 64.3 us at 8, 58.6 at 12; 960k: 435
+// and 425).
+// The damped neo-Hookean law alone also gains by that in the H8 adjoint and
+// one pass (step of 140k bricks 111.0 -> 106.8 us; 86.7 -> 92.4 without
+// damping). Not so the slab T10 operator product, which spills less: at 8
+// warps 62 us instead of 64.5 on 194k elements, but 267 instead of 254 on 960k.
 // T4, and H8 on the slab: 12 warps where the law's state fits 168 registers.
 // FP64 kernels take all 255 registers, and so do Q27 kernels (81-entry element
 // vectors; their shared-memory footprint limits the resident warps anyway).
@@ -390,10 +395,9 @@ template <int ET, typename R, int OP, bool AFF, int MAT> constexpr int min_ctas(
     if (h8_path<R>(ET, OP, AFF) && (OP == OP_FM || OP == OP_VJP) && MAT == MAT_NH_KV) return 2;
     if (t10_path<R>(ET, OP, AFF) || h8_path<R>(ET, OP, AFF)) return OP == OP_FORCE ? 4 : (MAT == MAT_ANY ? 2 : 3);
     if (OP == OP_VJP || OP == OP_FM) {
-        if (ET == ET_T10) return 2;
+        if (ET == ET_T10) return MAT == MAT_SVK ? 3 : 2;
         return ET == ET_T4 || MAT != MAT_ANY ? 3 : 2;
     }
-    if (OP == OP_MATVEC && !AFF && ET == ET_T10 && MAT == MAT_NH_KV) return 2;
     return (OP == OP_FORCE && AFF) ? 4 : 3;
 }
 
