@@ -67,26 +67,22 @@ WORKLOADS = {
            "neo-Hookean + Kelvin-Voigt, FP32",
 }
 GRAVITY = (0.0, 0.0, -9.81)
-# Algorithmic FP32 FLOPs per quadrature point of the neo-Hookean + Kelvin-Voigt
-# kernels on the affine path: T10 Q5 for the beam workload, Q27 for the q27
-# workload. force, matvec, vjp: 2 FFMA + FADD + FMUL thread instructions counted
-# by ncu on the scalar build of these kernels; force_matvec (the one-pass force +
-# operator product): 2 FFMA + FADD + FMUL + 4 FFMA2 + 2 FADD2 + 2 FMUL2 counted
-# by ncu on the packed build (the same count gives the adjoint 1820, against
-# 1786 on the scalar build)
-FLOP_PER_QP = {"beam": {"force": 852, "matvec": 1589, "vjp": 1786, "force_matvec": 1934},
-               "q27": {"force": 1932, "matvec": 3026, "vjp": 3567}}
+# FP32 FLOPs per quadrature point of the neo-Hookean + Kelvin-Voigt kernels on
+# the affine path: T10 Q5 for the beam workload, Q27 for the q27 workload:
+# 2 FFMA + FADD + FMUL + 4 FFMA2 + 2 FADD2 + 2 FMUL2 thread instructions counted
+# by ncu (profiles/element_kernels_counts.md). force_matvec: the one-pass force
+# + operator product
+FLOP_PER_QP = {"beam": {"force": 561, "matvec": 972, "vjp": 1089, "force_matvec": 1106},
+               "q27": {"force": 816, "matvec": 1348, "vjp": 1521}}
 # batch workload (affine path, no damping): FP32 FLOP per point by (element
-# type, law, op), law 0 = SVK, 1 = neo-Hookean; ncu counts of the per-law
-# kernels of one timed step (force, matvec: 2 FFMA + FADD + FMUL on the scalar
-# build, 512-body batch; force_matvec: with the packed instructions as above,
-# 64-body batch)
-FLOP_PER_QP_BATCH = {(0, 0): {"force": 288.3, "matvec": 503.3, "force_matvec": 652.3},
-                     (0, 1): {"force": 359.3, "matvec": 690.3, "force_matvec": 839.4},
-                     (1, 0): {"force": 483.7, "matvec": 865.7, "force_matvec": 1096.7},
-                     (1, 1): {"force": 552.3, "matvec": 1048.3, "force_matvec": 1279.3},
-                     (2, 0): {"force": 540.0, "matvec": 942.3, "force_matvec": 1188.5},
-                     (2, 1): {"force": 610.4, "matvec": 1124.7, "force_matvec": 1370.7}}
+# type, law, op), law 0 = SVK, 1 = neo-Hookean; the same counts of the per-law
+# kernels of a 64-body batch
+FLOP_PER_QP_BATCH = {(0, 0): {"force": 291.4, "matvec": 484.4, "force_matvec": 631.4},
+                     (0, 1): {"force": 389.3, "matvec": 676.4, "force_matvec": 823.3},
+                     (1, 0): {"force": 305.6, "matvec": 518.2, "force_matvec": 666.7},
+                     (1, 1): {"force": 404.5, "matvec": 711.9, "force_matvec": 860.7},
+                     (2, 0): {"force": 308.1, "matvec": 516.5, "force_matvec": 765.0},
+                     (2, 1): {"force": 404.0, "matvec": 777.2, "force_matvec": 955.2}}
 # how the end-to-end measurements move data
 OVERLAP = ("copies on their own streams: the next step's inputs are copied in while a step computes (two device "
            "staging sets), outputs are copied out as their operations end")
@@ -160,7 +156,7 @@ def peaks():
 # the mesh layout they read and their launch schedules (not the Newton,
 # constraint or load code): the committed ncu traffic is valid while these
 # are unchanged
-KERNEL_SOURCES = ("k_elem.cuh", "k_wpe.cuh", "k_fused.cuh", "tlfe_fused.h", "tlfe_elem.cuh", "tlfe_math.cuh",
+KERNEL_SOURCES = ("k_elem.cuh", "k_t10.cuh", "k_h8.cuh", "k_pw.cuh", "k_wpe.cuh", "k_fused.cuh", "tlfe_fused.h", "tlfe_elem.cuh", "tlfe_math.cuh",
                   "tlfe_internal.h", "tlfe_mesh.h", "api.cu", "k_setup.cu", "k_force.cu", "k_matvec.cu", "k_vjp.cu",
                   "k_diag.cu", "k_fm.cu", "k_fused_force.cu", "k_fused_matvec.cu")
 
